@@ -339,7 +339,7 @@ int fiona_linear_eval_level(const fiona_plan *plan, void *cuda_stream, uint32_t 
  * The last limb of every input poly is overwritten with r (r' when rounding); the other limbs
  * are only read.  `out` must not overlap `polys`.  Device pointers of the
  * ctx's device, 16-byte aligned.  Asynchronous on `cuda_stream`, except that
- * the first call on a ctx builds its twiddle tables (about 32 N L bytes of
+ * the first call on a ctx builds its twiddle tables (about 48 N L bytes of
  * device memory, held until fiona_ctx_destroy) synchronously: make it before
  * any stream capture.  Errors: FIONA_ERR_ARG (L_cur outside [2, L], null,
  * misaligned or overlapping buffers, unknown flags), FIONA_ERR_NODEVICE,

@@ -60,6 +60,7 @@ struct EncArgs {
     const int64_t *coeffs;  // [count][N]
     uint64_t *out;          // [count][Lc][N]
     const NttLimb *T;
+    uint32_t count;
     uint32_t Lc;
 };
 
@@ -86,8 +87,8 @@ __global__ void __launch_bounds__(LowPass<LN>::threads, 2) k_embed_low(EmbArgs A
     const double2 *z = A.slots + ((size_t)p << LN);
     const uint32_t *gat = A.E.gather + base;
     double2 *w = A.work + ((size_t)p << LN) + base;
-    inv_low_pass<LN>(
-        smem_raw, A.E.cinv, first, CplxArith{}, [&](uint32_t e) { return z[gat[e]]; },
+    inv_low_pass<LN, PS>(
+        smem_raw, A.E.cinv, first, CplxArith{}, 1, [&](uint32_t e0, uint32_t t) { return z[gat[e0 + t]]; },
         [&](uint32_t sub, uint32_t pos, double2 v) { w[(sub << PS::s) + pos] = v; });
 }
 
@@ -144,25 +145,33 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_enc_high(EncArgs
         [&](uint32_t sub, uint32_t pos, uint64_t v) { o[(size_t)pos * R2 + sub] = v; });
 }
 
-// RNS/NTT form, forward low stages, canonical store
+// RNS/NTT form, forward low stages, canonical store: the same rows of kPolys
+// polys per CTA (blockIdx.x = (group * Lc + limb) * tiles + tile)
 template <int LOGN, bool FAST>
-__global__ void __launch_bounds__(LowPass<LOGN>::threads, 4) k_enc_low(EncArgs A)
+__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 4) k_enc_low(EncArgs A)
 {
-    using SH = Shape<LOGN>;
-    using PS = LowPass<LOGN>;
+    using PS = LowPassPolys<LOGN>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), tr = blockIdx.x >> PS::ltiles;
-    const uint32_t l = tr % A.Lc;
-    const uint32_t first = tile << PS::lsubs;
-    uint64_t *o = A.out + ((size_t)tr << LOGN) + ((size_t)first << PS::s);
+    const uint32_t p0 = (tr / A.Lc) << PS::lpolys, l = tr % A.Lc;
+    const uint32_t first = tile << PS::lrows;
+    const size_t so = (size_t)A.Lc << LOGN;
+    uint64_t *o = A.out + p0 * so + ((size_t)l << LOGN) + ((size_t)first << PS::s);
+    const uint32_t np = A.count - p0;
     const NttLimb &Tl = A.T[l];
     const uint64_t q = Tl.q, mu = Tl.mu64;
-    fwd_low_pass<LOGN>(
-        smem_raw, Tl.fwd, first, ModArith<FAST>{q}, [] {},
-        [&](uint32_t sub, uint32_t pos) { return o[(sub << PS::s) + pos]; },
+    constexpr int le = PS::s + PS::lrows;  // log2 elements per poly
+    fwd_low_pass<LOGN, PS>(
+        smem_raw, Tl.fwd, first, ModArith<FAST>{q}, np, [] {},
+        [&](uint32_t sub, uint32_t pos) {
+            return o[(sub >> PS::lrows) * so + ((sub & (PS::rows - 1)) << PS::s) + pos];
+        },
         [&](auto t_of) {
-            sweep<PS, uint64_t>([&](uint32_t e) { return t_of(e); },
-                                [&](uint32_t e, uint64_t v) { o[e] = reduce_any(v, q, mu); });
+            sweep<PS, uint64_t>(
+                np, [&](uint32_t e0, uint32_t t) { return t_of(e0, t); },
+                [&](uint32_t e0, uint32_t t, uint64_t v) {
+                    o[(e0 >> le) * so + (e0 & ((1u << le) - 1)) + t] = reduce_any(v, q, mu);
+                });
         });
 }
 
@@ -182,11 +191,14 @@ int build_encode_tables(const fiona_ctx *ctx)
     double2 *tw = reinterpret_cast<double2 *>(host.data());
     double2 *twist = reinterpret_cast<double2 *>(host.data() + tw_bytes);
     uint32_t *gat = reinterpret_cast<uint32_t *>(host.data() + 2 * tw_bytes);
+    // the shape of the embedding's low pass (LowPass of log2 n)
+    const uint32_t n1 = ln / 2, lt = ln < (uint32_t)kLogTileMax ? ln : (uint32_t)kLogTileMax;
+    const uint32_t lrows = std::max(lt - 1, ln - n1) - (ln - n1);
     const long double pi = 3.141592653589793238462643383279502884L;
     for (uint32_t k = 0; k < n; ++k) {
         // psi^-brv(k) = zeta^(-2 brv(k)) and zeta^k, zeta = exp(i pi / N)
         const long double a = -2 * pi * (long double)bit_reverse(k, ln) / (long double)N;
-        tw[k] = make_double2((double)cosl(a), (double)sinl(a));
+        tw[low_place(k, n1, ln - n1, lrows)] = make_double2((double)cosl(a), (double)sinl(a));
         const long double b = pi * (long double)k / (long double)N;
         twist[k] = make_double2((double)cosl(b), (double)sinl(b));
     }
@@ -219,7 +231,7 @@ template <int LOGN>
 struct Inst {
     static constexpr size_t emb_low = LowPass<LOGN - 1>::template smem_bytes<CplxArith>();
     static constexpr size_t emb_high = HighPass<LOGN - 1>::template smem_bytes<CplxArith>();
-    static constexpr size_t enc_low = LowPass<LOGN>::template smem_bytes<ModArith<false>>();
+    static constexpr size_t enc_low = LowPassPolys<LOGN>::template smem_bytes<ModArith<false>>();
     static constexpr size_t enc_high = HighPass<LOGN>::template smem_bytes<ModArith<false>>();
 };
 
@@ -246,11 +258,11 @@ constexpr Kernels kernels_for()
                    LowPass<LOGN - 1>::ltiles,
                    HighPass<LOGN - 1>::ltiles,
                    HighPass<LOGN>::ltiles,
-                   LowPass<LOGN>::ltiles,
+                   LowPassPolys<LOGN>::ltiles,
                    LowPass<LOGN - 1>::threads,
                    HighPass<LOGN - 1>::threads,
                    HighPass<LOGN>::threads,
-                   LowPass<LOGN>::threads};
+                   LowPassPolys<LOGN>::threads};
 }
 
 const Kernels &kernels(uint32_t n)
@@ -343,9 +355,10 @@ int launch_encode_coeffs(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64
         const uint64_t np = std::min<uint64_t>(count - p0, max_polys);
         a.coeffs = coeffs + p0 * ctx->N;
         a.out = out + p0 * Lc * (uint64_t)ctx->N;
-        const uint64_t nt = np * Lc;
+        a.count = (uint32_t)np;
+        const uint64_t nt = np * Lc, ng = (np + kPolys - 1) / kPolys;
         K.enc_high[fast]<<<(uint32_t)(nt << K.lt_enc_high), K.t_enc_high, K.s_enc_high, s>>>(a);
-        K.enc_low[fast]<<<(uint32_t)(nt << K.lt_enc_low), K.t_enc_low, K.s_enc_low, s>>>(a);
+        K.enc_low[fast]<<<(uint32_t)((ng * Lc) << K.lt_enc_low), K.t_enc_low, K.s_enc_low, s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "encode launch: %s", cudaGetErrorString(e));

@@ -74,7 +74,7 @@ double rate(int sms, const uint64_t *seed, uint64_t *sink)
 }
 
 // Forward NTT butterflies of the rescale (fiona_ntt::ModArith::ct: one
-// product by a twiddle with Shoup's precomputed quotient, a sum and a
+// product by a twiddle with its precomputed quotients, a sum and a
 // difference), FAST = without the conditional subtraction (every modulus
 // below 2^56), in kChains independent chains per thread; the twiddle changes
 // every step so that nothing folds away.
@@ -83,23 +83,24 @@ __global__ void __launch_bounds__(256) bfly_kernel(const uint64_t *seed, uint64_
 {
     const fiona_ntt::ModArith<FAST> ar{(seed[0] >> 14) | 1};
     uint64_t x[kChains], y[kChains];
-    ulonglong2 w[kChains];
+    fiona_ntt::Twiddle w[kChains];
 #pragma unroll
     for (int c = 0; c < kChains; ++c) {
         x[c] = seed[(threadIdx.x + c) & 63] >> 14;
         y[c] = seed[(threadIdx.x + 7 * c + 1) & 63] >> 14;
-        w[c] = make_ulonglong2(seed[(threadIdx.x + 3 * c + 2) & 63] >> 14, seed[(threadIdx.x + 5 * c + 3) & 63]);
+        w[c].wv = make_ulonglong2(seed[(threadIdx.x + 3 * c + 2) & 63] >> 14, seed[(threadIdx.x + 5 * c + 3) & 63] >> 14);
+        w[c].om = make_uint2((uint32_t)(seed[(threadIdx.x + c + 4) & 63] >> 33), (uint32_t)(seed[(threadIdx.x + c + 5) & 63] >> 33));
     }
     for (int s = 0; s < kSteps; ++s) {
 #pragma unroll
         for (int c = 0; c < kChains; ++c) {
             ar.ct(x[c], y[c], w[c]);
-            w[c].x ^= y[c] & 0xF;
+            w[c].wv.x ^= y[c] & 0xF;
         }
     }
     uint64_t r = 0;
 #pragma unroll
-    for (int c = 0; c < kChains; ++c) r += x[c] ^ y[c] ^ w[c].x;
+    for (int c = 0; c < kChains; ++c) r += x[c] ^ y[c] ^ w[c].wv.x;
     sink[blockIdx.x * blockDim.x + threadIdx.x] = r;
 }
 

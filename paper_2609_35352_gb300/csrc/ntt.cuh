@@ -19,9 +19,10 @@
 //              tile / R1 of them (adjacent columns, so accesses coalesce);
 //   low pass   the other stages, inside blocks of R2 consecutive elements;
 //              a CTA takes tile / R2 blocks.
-// A CTA's tile is 4096 elements in the high pass and 2048 in the low pass
-// (whose CTAs also stage about one twiddle per element: the smaller tile lets
-// more CTAs share an SM); a thread handles 16 elements.
+// A CTA's tile is 4096 elements in the high pass; in the low pass, whose CTAs
+// also stage about one twiddle per element, it is the same rows of eight polys
+// (4096 elements, 512 twiddles) for the transforms mod q and 2048 elements of
+// one for the complex ones.  A thread handles 16 elements.
 // A pass runs its stages in rounds of up to 4: in a round each thread holds
 // the 2^K elements of one group in registers, spaced by the round's smallest
 // distance, and applies the round's K stages to them (a group needs 2^K - 1
@@ -37,29 +38,34 @@
 
 namespace fiona_ntt {
 
-constexpr int kLogTileMax = 12;  // at most 4096 elements per CTA (2048 in the low pass)
+constexpr int kLogTileMax = 12;  // at most 4096 elements per CTA
 constexpr int kLogNMin = 10, kLogNMax = 17;  // the ring dimensions a context accepts
 
-// ---------------------------------------------------------------------------
-// Residues mod q < 2^60 in 64-bit words.  A product by a table constant w
-// uses Shoup's precomputed w' = floor(w 2^64 / q): r = x w - floor(x w' /
-// 2^64) q lies in [0, 2q) for any 64-bit x.  The quotient is taken from
-// three of the four 32-bit partial products of x w' (the low-by-low one and
-// the carries below bit 64 are dropped), which underestimates it by at most
-// 2, so r lies in [0, 4q).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t mul_shoup_lazy(uint64_t x, ulonglong2 w, uint64_t q)
+// B bytes (16, or 8) global -> shared, asynchronous
+template <int B>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem)
 {
-    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32);
-    const uint32_t wl = (uint32_t)w.y, wh = (uint32_t)(w.y >> 32);
-    const uint64_t qh = (uint64_t)xh * wh + __umulhi(xh, wl) + __umulhi(xl, wh);
-    return x * w.x + qh * (0 - q);
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+    if constexpr (B == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-__device__ __forceinline__ uint64_t csub(uint64_t x, uint64_t c) { return x >= c ? x - c : x; }
+// ---------------------------------------------------------------------------
+// Residues mod q < 2^60 in 64-bit words.
+// ---------------------------------------------------------------------------
+// x - c if that is not negative, else x (x - c within a signed word: every
+// use has x, c < 12q and |x - c| < 7q < 2^63; the sign is one test of the
+// high half)
+__device__ __forceinline__ uint64_t csub(uint64_t x, uint64_t c)
+{
+    const int64_t d = (int64_t)(x - c);
+    return d < 0 ? x : (uint64_t)d;
+}
 
-// x in [0, 4q) -> canonical
-__device__ __forceinline__ uint64_t canon4(uint64_t x, uint64_t q) { return csub(csub(x, 2 * q), q); }
+// x in [0, 6q) -> canonical
+__device__ __forceinline__ uint64_t canon6(uint64_t x, uint64_t q) { return csub(csub(csub(x, 4 * q), 2 * q), q); }
 
 // x mod q for any 64-bit x: floor(x * mu64 / 2^64), mu64 = floor(2^64 / q),
 // is floor(x / q) or one less
@@ -68,31 +74,99 @@ __device__ __forceinline__ uint64_t reduce_any(uint64_t x, uint64_t q, uint64_t 
     return csub(x - __umul64hi(x, mu64) * q, q);
 }
 
+// A constant w of a limb (a twiddle, N^-1, q_j^-1): w and v = w 2^32 mod q,
+// and their quotients by 2q, om = floor(2^32 w / 2q) and ov = floor(2^32 v /
+// 2q), both below 2^31.
+struct __align__(16) Twiddle {
+    ulonglong2 wv;  // (w, v)
+    uint2 om;       // (om, ov)
+};
+struct TwiddleTable {  // a limb's table in global memory
+    const ulonglong2 *wv;
+    const uint2 *om;
+};
+struct TwiddleStage {  // a pass's twiddles in shared memory
+    ulonglong2 *wv;
+    uint2 *om;
+    __device__ __forceinline__ Twiddle operator[](uint32_t i) const { return Twiddle{wv[i], om[i]}; }
+};
+
+// x * w mod q for any 64-bit x = xh 2^32 + xl, lazily: V = xl w + xh v is
+// congruent to x w; with k = floor((xl om + xh ov) / 2^32),
+//   V / 2q - 3 < k <= V / 2q
+// (om and ov fall short of their exact values by less than 1 each, so the
+// sum by less than xl + xh < 2^33; the floor takes less than 1 more), and
+// r = V - k 2q, computed modulo 2^64, lies in [0, 6q), below 2^63.  The sum
+// does not wrap (each product is below 2^63), and k fits in 32 bits: that is
+// what the quotient by 2q is for.
+// Five 32x32 -> 64-bit products and three 32-bit ones.  Shoup's product with
+// one precomputed quotient floor(2^64 w / q) takes five (two of them for the
+// high half only) and four.  The FMA-heavy pipe bounds every transform here,
+// and on sm_103a a 64-bit product holds it for 4 cycles a warp, a 32-bit one
+// for 2.  Measured in a register-only chain of radix-16 groups (GB300, 16
+// warps an SM): 36.0 cycles a butterfly and warp scheduler against 42.4, the
+// pipe 85-89% busy in both.  The product by k is added last and by itself:
+// with the three wide products in one chain of multiply-adds it measured
+// 39.7; written without the explicit word operations, 37-40.
+__device__ __forceinline__ uint64_t mul_twiddle(uint64_t x, const Twiddle &t, uint64_t q)
+{
+    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32);
+    const uint64_t n = 0 - 2 * q;
+    uint64_t m, p, k2, r;
+    uint32_t hi;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(m) : "r"(xl), "r"(t.om.x));
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(m) : "r"(xh), "r"(t.om.y));
+    const uint32_t k = (uint32_t)(m >> 32);
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(xl), "r"((uint32_t)t.wv.x));
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(p) : "r"(xh), "r"((uint32_t)t.wv.y));
+    hi = (uint32_t)(p >> 32);
+    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(hi) : "r"(xl), "r"((uint32_t)(t.wv.x >> 32)));
+    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(hi) : "r"(xh), "r"((uint32_t)(t.wv.y >> 32)));
+    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(hi) : "r"(k), "r"((uint32_t)(n >> 32)));
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(k2) : "r"(k), "r"((uint32_t)n));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"((uint32_t)p), "r"(hi));
+    return r + k2;
+}
+
 // Modular butterflies.  Values between stages:
-//   forward, general   in [0, 8q): x is brought below 4q before each
-//                      butterfly (x + t, x - t + 4q with t in [0, 4q));
-//   forward, FAST      (q < 2^56, inputs below 5q) no reduction at all: each
-//                      stage adds less than 4q to the bound, so after at most
-//                      17 stages values stay below 73q < 2^63;
-//   inverse            in [0, 4q): x + y is brought below 4q, and
-//                      x - y + 4q is only multiplied.
+//   forward, general   in [0, 12q): x is brought below 6q before each
+//                      butterfly (x + t, x - t + 6q with t in [0, 6q));
+//   forward, FAST      (q < 2^56, inputs below 8q) no reduction at all: each
+//                      stage adds less than 6q to the bound, so after at most
+//                      17 stages values stay below 110q < 2^63;
+//   inverse            in [0, 6q): x + y is brought below 6q, and
+//                      x - y + 6q is only multiplied.
+// A pass stages its twiddles in shared memory as two arrays (16 and 8 bytes
+// an entry).
 template <bool FAST>
 struct ModArith {
     typedef uint64_t T;
-    typedef ulonglong2 W;  // (w, Shoup companion)
-    uint64_t q;
-    __device__ __forceinline__ void ct(T &x, T &y, W w) const
+    typedef Twiddle W;
+    static constexpr size_t w_bytes = 24;
+    typedef TwiddleTable Table;
+    typedef TwiddleStage Staged;
+    __device__ __forceinline__ static Staged staged(uint8_t *raw, int entries)
     {
-        const uint64_t a = FAST ? x : csub(x, 4 * q);
-        const uint64_t t = mul_shoup_lazy(y, w, q);
-        x = a + t;
-        y = a + 4 * q - t;
+        return Staged{reinterpret_cast<ulonglong2 *>(raw), reinterpret_cast<uint2 *>(raw + 16 * (size_t)entries)};
     }
-    __device__ __forceinline__ void gs(T &x, T &y, W w) const
+    __device__ __forceinline__ static void stage(const Staged &s, uint32_t i, const Table &t, uint32_t k)
+    {
+        cp_async<16>(&s.wv[i], &t.wv[k]);
+        cp_async<8>(&s.om[i], &t.om[k]);
+    }
+    uint64_t q;
+    __device__ __forceinline__ void ct(T &x, T &y, const W &w) const
+    {
+        const uint64_t a = FAST ? x : csub(x, 6 * q);
+        const uint64_t t = mul_twiddle(y, w, q);
+        x = a + t;
+        y = a + 6 * q - t;
+    }
+    __device__ __forceinline__ void gs(T &x, T &y, const W &w) const
     {
         const uint64_t a = x, b = y;
-        x = csub(a + b, 4 * q);
-        y = mul_shoup_lazy(a + 4 * q - b, w, q);
+        x = csub(a + b, 6 * q);
+        y = mul_twiddle(a + 6 * q - b, w, q);
     }
 };
 
@@ -100,6 +174,11 @@ struct ModArith {
 struct CplxArith {
     typedef double2 T;
     typedef double2 W;
+    static constexpr size_t w_bytes = 16;
+    typedef const double2 *Table;
+    typedef double2 *Staged;
+    __device__ __forceinline__ static Staged staged(uint8_t *raw, int) { return reinterpret_cast<double2 *>(raw); }
+    __device__ __forceinline__ static void stage(Staged s, uint32_t i, Table t, uint32_t k) { cp_async<16>(&s[i], &t[k]); }
     __device__ __forceinline__ static double2 mul(double2 a, double2 b)
     {
         return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
@@ -130,9 +209,13 @@ struct Shape {
 
 // A pass over a tile: 2^LSUBS sub-transforms of 2^S positions, in rounds,
 // 2^LTILES tiles per transform, 16 elements per thread (at least 64 threads).
-template <int S, int LSUBS, bool HIGH, int LTILES>
+// With LPOLYS > 0 (low pass) the sub-transforms are the same 2^lrows rows of
+// 2^LPOLYS polys: sub = poly << lrows | row, and the polys share their
+// twiddles.
+template <int S, int LSUBS, bool HIGH, int LTILES, int LPOLYS = 0>
 struct PassShape {
     static constexpr int s = S, lsubs = LSUBS, subs = 1 << LSUBS;
+    static constexpr int lpolys = LPOLYS, polys = 1 << LPOLYS, lrows = LSUBS - LPOLYS, rows = 1 << lrows;
     static constexpr int tile = 1 << (S + LSUBS);
     static constexpr int ltiles = LTILES;
     static constexpr uint32_t threads = tile / 16 < 64 ? 64 : tile / 16;
@@ -142,12 +225,13 @@ struct PassShape {
     __host__ __device__ static constexpr int J0(int r) { return r == 0 ? 0 : J0(r - 1) + K(r - 1); }
     static constexpr bool high = HIGH;
     // shared memory: the staged twiddles (2^s entries for the high pass, at
-    // most one per tile element for the low pass), then the padded tile
-    static constexpr int tw_entries = HIGH ? 1 << S : 1 << (S + LSUBS);
+    // most one per element of a poly's rows for the low pass), then the
+    // padded tile
+    static constexpr int tw_entries = HIGH ? 1 << S : 1 << (S + lrows);
     template <class A>
     __host__ __device__ static constexpr size_t smem_bytes()
     {
-        return sizeof(typename A::W) * tw_entries + sizeof(typename A::T) * subs * pitch;
+        return A::w_bytes * tw_entries + sizeof(typename A::T) * subs * pitch;
     }
 };
 
@@ -161,6 +245,18 @@ struct LowShape {
 };
 template <int LOGN>
 using LowPass = PassShape<LowShape<LOGN>::s, LowShape<LOGN>::lt - LowShape<LOGN>::s, false, LOGN - LowShape<LOGN>::lt>;
+
+// The low pass of several polys at once (the transforms mod q): a tile of
+// 4096 elements, kPolys polys of 4096 / kPolys.  A low-pass CTA needs one
+// twiddle (24 bytes) per element of its rows, read through L2 and staged by
+// its threads; sharing them between the polys of a batch divides both that
+// traffic and its instructions by kPolys, and leaves room for 32 warps an SM
+// (45 KB a CTA of 256 threads).  Measured on GB300, 192 polys of 2^16, 12
+// limbs: the rescale 1.488 ms with 4 polys a CTA, 1.410 with 8.
+constexpr int kLogPolys = 3, kPolys = 1 << kLogPolys;
+template <int LOGN>
+using LowPassPolys = PassShape<LOGN - Shape<LOGN>::n1, kLogTileMax - (LOGN - Shape<LOGN>::n1), false,
+                               LOGN - kLogTileMax + kLogPolys, kLogPolys>;
 
 // Group g of round R: sub-transform `sub`, and the element positions
 // (hi << (lD + K)) + (i << lD) + lo, i < 2^K.  High pass: sub-transforms
@@ -191,13 +287,13 @@ struct Group {
     {
         const int j = J0 + k;
         if (PS::high) return (1u << j) + (hi << k) + b;
-        return ((PS::subs << j) - PS::subs) + (((hi << k) + b) << PS::lsubs) + sub;
+        return ((PS::rows << j) - PS::rows) + (((hi << k) + b) << PS::lrows) + (sub & (PS::rows - 1));
     }
 };
 
 template <class PS, int R, int k, bool INV, class A>
 __device__ __forceinline__ void group_stage(typename A::T (&x)[1 << PS::K(R)], const Group<PS, R> &G,
-                                            const typename A::W *stw, const A &ar)
+                                            const typename A::Staged &stw, const A &ar)
 {
     constexpr int K = PS::K(R), h = 1 << (K - 1 - k);
 #pragma unroll
@@ -215,7 +311,7 @@ __device__ __forceinline__ void group_stage(typename A::T (&x)[1 << PS::K(R)], c
 
 template <class PS, int R, bool INV, class A>
 __device__ __forceinline__ void group_stages(typename A::T (&x)[1 << PS::K(R)], const Group<PS, R> &G,
-                                             const typename A::W *stw, const A &ar)
+                                             const typename A::Staged &stw, const A &ar)
 {
     constexpr int K = PS::K(R);
     if constexpr (!INV) {
@@ -231,11 +327,21 @@ __device__ __forceinline__ void group_stages(typename A::T (&x)[1 << PS::K(R)], 
     }
 }
 
+// Whether sub-transform `sub` is one of the `np` polys a CTA has (the last
+// group of a batch may have fewer than PS::polys: their rows take part in
+// nothing).
+template <class PS>
+__device__ __forceinline__ bool present(uint32_t sub, uint32_t np)
+{
+    return PS::lpolys == 0 || (sub >> PS::lrows) < np;
+}
+
 // One round: every group of this thread is loaded (ld(sub, pos)), then
 // `between()` runs (once, on every thread), then the groups are transformed
 // and stored (st(sub, pos, value)).
 template <class PS, int R, bool INV, class A, class Ld, class Between, class St>
-__device__ __forceinline__ void round(const typename A::W *stw, const A &ar, Ld ld, Between between, St st)
+__device__ __forceinline__ void round(const typename A::Staged &stw, const A &ar, uint32_t np, Ld ld, Between between,
+                                      St st)
 {
     using Gr = Group<PS, R>;
     constexpr int P = Gr::per_thread, E = 1 << Gr::K;
@@ -245,8 +351,9 @@ __device__ __forceinline__ void round(const typename A::W *stw, const A &ar, Ld 
         const uint32_t g = threadIdx.x + gi * PS::threads;
         if (Gr::groups % PS::threads == 0 || g < Gr::groups) {
             const Gr G(g);
+            if (present<PS>(G.sub, np))
 #pragma unroll
-            for (int i = 0; i < E; ++i) x[gi][i] = ld(G.sub, G.pos(i));
+                for (int i = 0; i < E; ++i) x[gi][i] = ld(G.sub, G.pos(i));
         }
     }
     between();
@@ -255,56 +362,60 @@ __device__ __forceinline__ void round(const typename A::W *stw, const A &ar, Ld 
         const uint32_t g = threadIdx.x + gi * PS::threads;
         if (Gr::groups % PS::threads == 0 || g < Gr::groups) {
             const Gr G(g);
-            group_stages<PS, R, INV>(x[gi], G, stw, ar);
+            if (present<PS>(G.sub, np)) {
+                group_stages<PS, R, INV>(x[gi], G, stw, ar);
 #pragma unroll
-            for (int i = 0; i < E; ++i) st(G.sub, G.pos(i), x[gi][i]);
+                for (int i = 0; i < E; ++i) st(G.sub, G.pos(i), x[gi][i]);
+            }
         }
     }
 }
 
 // the rounds from R up to (excluding) REND, through shared memory
 template <class PS, int R, int REND, bool INV, class A>
-__device__ __forceinline__ void middle_rounds(typename A::T *sm, const typename A::W *stw, const A &ar)
+__device__ __forceinline__ void middle_rounds(typename A::T *sm, const typename A::Staged &stw, const A &ar, uint32_t np)
 {
     if constexpr (R != REND) {
         round<PS, R, INV>(
-            stw, ar, [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; }, [] {},
+            stw, ar, np, [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; }, [] {},
             [&](uint32_t sub, uint32_t pos, typename A::T v) { sm[sub * PS::pitch + pos] = v; });
         __syncthreads();
-        middle_rounds<PS, (INV ? R - 1 : R + 1), REND, INV>(sm, stw, ar);
+        middle_rounds<PS, (INV ? R - 1 : R + 1), REND, INV>(sm, stw, ar, np);
     }
 }
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+// The tables.  Entry k >= 1 of a transform's twiddles is psi^brv(k) (forward)
+// or psi^-brv(k) (inverse); the stage with m blocks uses entries m .. 2m - 1.
+// The high pass needs entries [0, R1): the entry of its local stage j for
+// position pos is 2^j + (pos >> (s - j)), for every sub-transform.  Row `row`
+// of the low pass needs ((R1 + row) << j) + t for its local stages j < s and
+// t < 2^j, each entry of [R1, N) used by one row; they are stored in the
+// order in which a CTA stages them, so that staging is a plain copy: the
+// rows of a CTA's tile together, stage j's entries from (rows << j) - rows
+// on, t-major ([t][row]: adjacent rows read adjacent words of shared memory).
+// (With the entries at their index k and the order made while staging, that
+// took 27% of the forward low pass's instructions.)  low_place is the place of
+// entry k for tiles of 2^lrows rows.
+inline uint32_t low_place(uint32_t k, uint32_t n1, uint32_t s, uint32_t lrows)
 {
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+    if (k >> n1 == 0) return k;
+    uint32_t j = 0;
+    while (k >> (n1 + j + 1)) ++j;
+    const uint32_t row = (k >> j) - (1u << n1), t = k & ((1u << j) - 1);
+    const uint32_t tile = row >> lrows, r = row & ((1u << lrows) - 1);
+    return (1u << n1) + ((tile * ((1u << s) - 1)) << lrows) + (((1u << j) - 1) << lrows) + (t << lrows) + r;
 }
 
-// Stage the pass's twiddles (cp.async; waited by wait_twiddles).  `tab` is
-// the transform's table: entry k is psi^brv(k) (forward) or psi^-brv(k)
-// (inverse), 16 bytes each.
-//   high pass  the entry of local stage j for position pos is 2^j + (pos >>
-//              (s - j)) for every sub-transform: entries [0, 2^s) are copied;
-//   low pass   sub-transform `sub` is row first + sub of the poly and its
-//              entry is ((R1 + first + sub) << j) + t, t < 2^j; stage j's
-//              entries are stored from (subs << j) - subs, t-major
-//              ([t][sub]), so that adjacent sub-transforms read adjacent words.
-template <int LOGN, class PS, class W>
-__device__ __forceinline__ void stage_twiddles(W *stw, const W *tab, uint32_t first)
+// Stage the pass's twiddles (cp.async; waited by wait_twiddles); `first` is
+// the low pass's first row
+template <int LOGN, class PS, class A>
+__device__ __forceinline__ void stage_twiddles(const typename A::Staged &stw, const typename A::Table &tab, uint32_t first)
 {
-    static_assert(sizeof(W) == 16, "twiddles are copied in 16-byte units");
-    if constexpr (PS::high) {
-        for (uint32_t e = threadIdx.x; e < (1u << PS::s); e += PS::threads) cp_async16(&stw[e], &tab[e]);
-    } else {
-        const uint32_t u = (1u << Shape<LOGN>::n1) + first;
-#pragma unroll 1
-        for (int j = 0; j < PS::s; ++j) {
-            const uint32_t cnt = PS::subs << j, off = cnt - PS::subs;
-            for (uint32_t e = threadIdx.x; e < cnt; e += PS::threads)
-                cp_async16(&stw[off + ((e & ((1u << j) - 1)) << PS::lsubs) + (e >> j)], &tab[(u << j) + e]);
-        }
-    }
+    constexpr uint32_t cnt = PS::high ? 1u << PS::s : (uint32_t)PS::rows * ((1u << PS::s) - 1);
+    const uint32_t base = PS::high ? 0 : (1u << Shape<LOGN>::n1) + first * ((1u << PS::s) - 1);
+#pragma unroll
+    for (uint32_t e = 0; e < cnt; e += PS::threads)
+        if (e + PS::threads <= cnt || e + threadIdx.x < cnt) A::stage(stw, e + threadIdx.x, tab, base + e + threadIdx.x);
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
@@ -314,133 +425,149 @@ __device__ __forceinline__ void wait_twiddles()
     __syncthreads();
 }
 
-// A coalesced sweep over the tile's elements e (tile / threads per thread):
-// every load first, then every store.
+// the same for the element e0 + t of a sweep below (a poly's rows are a
+// multiple of the threads)
+template <class PS>
+__device__ __forceinline__ bool has(uint32_t e0, uint32_t np)
+{
+    static_assert(PS::lpolys == 0 || (1 << (PS::s + PS::lrows)) % PS::threads == 0, "whole steps per poly");
+    return PS::lpolys == 0 || (e0 >> (PS::s + PS::lrows)) < np;
+}
+
+// A coalesced sweep over the tile's elements e = e0 + t (tile / threads per
+// thread; e0 a constant multiple of the thread count, t the thread): every
+// load first, then every store.
 template <class PS, class T, class Ld, class St>
-__device__ __forceinline__ void sweep(Ld ld, St st)
+__device__ __forceinline__ void sweep(uint32_t np, Ld ld, St st)
 {
     constexpr int P = (PS::tile + (int)PS::threads - 1) / (int)PS::threads;
     T v[P];
 #pragma unroll
-    for (int i = 0; i < P; ++i) {
-        const uint32_t e = threadIdx.x + i * PS::threads;
-        if (PS::tile % PS::threads == 0 || e < PS::tile) v[i] = ld(e);
-    }
+    for (int i = 0; i < P; ++i)
+        if ((PS::tile % PS::threads == 0 || threadIdx.x + i * PS::threads < PS::tile) && has<PS>(i * PS::threads, np))
+            v[i] = ld(i * PS::threads, threadIdx.x);
 #pragma unroll
-    for (int i = 0; i < P; ++i) {
-        const uint32_t e = threadIdx.x + i * PS::threads;
-        if (PS::tile % PS::threads == 0 || e < PS::tile) st(e, v[i]);
-    }
+    for (int i = 0; i < P; ++i)
+        if ((PS::tile % PS::threads == 0 || threadIdx.x + i * PS::threads < PS::tile) && has<PS>(i * PS::threads, np))
+            st(i * PS::threads, threadIdx.x, v[i]);
+}
+
+// the padded position of element e0 + t of a tile in shared memory
+template <class PS>
+__device__ __forceinline__ uint32_t padded(uint32_t e0, uint32_t t)
+{
+    if constexpr (PS::threads % (1u << PS::s) == 0)  // whole rows per step
+        return ((e0 >> PS::s) + (t >> PS::s)) * PS::pitch + (t & ((1u << PS::s) - 1));
+    else
+        return ((e0 + t) >> PS::s) * PS::pitch + ((e0 + t) & ((1u << PS::s) - 1));
 }
 
 // shared memory of a pass: staged twiddles, then the tile
 template <class PS, class A>
 struct Smem {
-    typename A::W *stw;
+    typename A::Staged stw;
     typename A::T *sm;
     __device__ __forceinline__ explicit Smem(uint8_t *raw)
-        : stw(reinterpret_cast<typename A::W *>(raw)), sm(reinterpret_cast<typename A::T *>(stw + PS::tw_entries))
+        : stw(A::staged(raw, PS::tw_entries)),
+          sm(reinterpret_cast<typename A::T *>(raw + A::w_bytes * PS::tw_entries))
     {
     }
 };
 
 // ---------------------------------------------------------------------------
 // Pass drivers.  `first` is the tile's first column (high) or row (low);
-// the callbacks address the tile by (sub, pos), or by the element index e of
-// a coalesced sweep, in which poly index = first * R2 + e (low pass).
+// the callbacks address the tile by (sub, pos), or by the element index e =
+// sub * 2^s + pos of a coalesced sweep.  Low passes take the pass shape and
+// the polys the CTA has.
 // ---------------------------------------------------------------------------
 
 // forward high pass: the first round loads directly (gload), the last stores
 // directly (gstore)
 template <int LOGN, class A, class GLoad, class GStore>
-__device__ __forceinline__ void fwd_high_pass(uint8_t *raw, const typename A::W *tab, uint32_t first, const A &ar,
+__device__ __forceinline__ void fwd_high_pass(uint8_t *raw, const typename A::Table &tab, uint32_t first, const A &ar,
                                               GLoad gload, GStore gstore)
 {
     using PS = HighPass<LOGN>;
     Smem<PS, A> S(raw);
     typename A::T *sm = S.sm;
-    stage_twiddles<LOGN, PS>(S.stw, tab, first);
+    stage_twiddles<LOGN, PS, A>(S.stw, tab, first);
     auto sload = [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; };
     auto sstore = [&](uint32_t sub, uint32_t pos, typename A::T v) { sm[sub * PS::pitch + pos] = v; };
     if constexpr (PS::nr == 1) {
-        round<PS, 0, false>(S.stw, ar, gload, wait_twiddles, gstore);
+        round<PS, 0, false>(S.stw, ar, 1, gload, wait_twiddles, gstore);
     } else {
-        round<PS, 0, false>(S.stw, ar, gload, wait_twiddles, sstore);
+        round<PS, 0, false>(S.stw, ar, 1, gload, wait_twiddles, sstore);
         __syncthreads();
-        middle_rounds<PS, 1, PS::nr - 1, false>(sm, S.stw, ar);
-        round<PS, PS::nr - 1, false>(S.stw, ar, sload, [] {}, gstore);
+        middle_rounds<PS, 1, PS::nr - 1, false>(sm, S.stw, ar, 1);
+        round<PS, PS::nr - 1, false>(S.stw, ar, 1, sload, [] {}, gstore);
     }
 }
 
 // forward low pass: the first round (lo fastest) loads directly; the last
-// round goes through shared memory to a coalesced sweep epi(e, value), every
+// round goes through shared memory to a coalesced sweep epi(value of e0, t), every
 // value read by then (`pre()` runs before the first round)
-template <int LOGN, class A, class Pre, class GLoad, class Epi>
-__device__ __forceinline__ void fwd_low_pass(uint8_t *raw, const typename A::W *tab, uint32_t first, const A &ar,
-                                             Pre pre, GLoad gload, Epi epi)
+template <int LOGN, class PS, class A, class Pre, class GLoad, class Epi>
+__device__ __forceinline__ void fwd_low_pass(uint8_t *raw, const typename A::Table &tab, uint32_t first, const A &ar,
+                                             uint32_t np, Pre pre, GLoad gload, Epi epi)
 {
-    using PS = LowPass<LOGN>;
     Smem<PS, A> S(raw);
     typename A::T *sm = S.sm;
-    stage_twiddles<LOGN, PS>(S.stw, tab, first);
+    stage_twiddles<LOGN, PS, A>(S.stw, tab, first);
     pre();
     auto sstore = [&](uint32_t sub, uint32_t pos, typename A::T v) { sm[sub * PS::pitch + pos] = v; };
-    round<PS, 0, false>(S.stw, ar, gload, wait_twiddles, sstore);
+    round<PS, 0, false>(S.stw, ar, np, gload, wait_twiddles, sstore);
     __syncthreads();
-    middle_rounds<PS, 1, PS::nr, false>(sm, S.stw, ar);
-    epi([&](uint32_t e) { return sm[(e >> PS::s) * PS::pitch + (e & ((1u << PS::s) - 1))]; });
+    middle_rounds<PS, 1, PS::nr, false>(sm, S.stw, ar, np);
+    epi([&](uint32_t e0, uint32_t t) { return sm[padded<PS>(e0, t)]; });
 }
 
-// inverse low pass: a coalesced sweep in (sweep_load(e)), the rounds, the
+// inverse low pass: a coalesced sweep in (sweep_load(e0, t)), the rounds, the
 // last round (lo fastest) stores directly
-template <int LOGN, class A, class SLoad, class GStore>
-__device__ __forceinline__ void inv_low_pass(uint8_t *raw, const typename A::W *tab, uint32_t first, const A &ar,
-                                             SLoad sweep_load, GStore gstore)
+template <int LOGN, class PS, class A, class SLoad, class GStore>
+__device__ __forceinline__ void inv_low_pass(uint8_t *raw, const typename A::Table &tab, uint32_t first, const A &ar,
+                                             uint32_t np, SLoad sweep_load, GStore gstore)
 {
-    using PS = LowPass<LOGN>;
     Smem<PS, A> S(raw);
     typename A::T *sm = S.sm;
-    stage_twiddles<LOGN, PS>(S.stw, tab, first);
-    sweep<PS, typename A::T>(sweep_load, [&](uint32_t e, typename A::T v) {
-        sm[(e >> PS::s) * PS::pitch + (e & ((1u << PS::s) - 1))] = v;
-    });
+    stage_twiddles<LOGN, PS, A>(S.stw, tab, first);
+    sweep<PS, typename A::T>(np, sweep_load, [&](uint32_t e0, uint32_t t, typename A::T v) { sm[padded<PS>(e0, t)] = v; });
     wait_twiddles();
-    middle_rounds<PS, PS::nr - 1, 0, true>(sm, S.stw, ar);
+    middle_rounds<PS, PS::nr - 1, 0, true>(sm, S.stw, ar, np);
     round<PS, 0, true>(
-        S.stw, ar, [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; }, [] {}, gstore);
+        S.stw, ar, np, [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; }, [] {}, gstore);
 }
 
 // inverse high pass: the first round (sub-transforms fastest) loads
 // directly, the last stores directly
 template <int LOGN, class A, class GLoad, class GStore>
-__device__ __forceinline__ void inv_high_pass(uint8_t *raw, const typename A::W *tab, uint32_t first, const A &ar,
+__device__ __forceinline__ void inv_high_pass(uint8_t *raw, const typename A::Table &tab, uint32_t first, const A &ar,
                                               GLoad gload, GStore gstore)
 {
     using PS = HighPass<LOGN>;
     Smem<PS, A> S(raw);
     typename A::T *sm = S.sm;
-    stage_twiddles<LOGN, PS>(S.stw, tab, first);
+    stage_twiddles<LOGN, PS, A>(S.stw, tab, first);
     auto sload = [&](uint32_t sub, uint32_t pos) { return sm[sub * PS::pitch + pos]; };
     auto sstore = [&](uint32_t sub, uint32_t pos, typename A::T v) { sm[sub * PS::pitch + pos] = v; };
     if constexpr (PS::nr == 1) {
-        round<PS, 0, true>(S.stw, ar, gload, wait_twiddles, gstore);
+        round<PS, 0, true>(S.stw, ar, 1, gload, wait_twiddles, gstore);
     } else {
-        round<PS, PS::nr - 1, true>(S.stw, ar, gload, wait_twiddles, sstore);
+        round<PS, PS::nr - 1, true>(S.stw, ar, 1, gload, wait_twiddles, sstore);
         __syncthreads();
-        middle_rounds<PS, PS::nr - 2, 0, true>(sm, S.stw, ar);
-        round<PS, 0, true>(S.stw, ar, sload, [] {}, gstore);
+        middle_rounds<PS, PS::nr - 2, 0, true>(sm, S.stw, ar, 1);
+        round<PS, 0, true>(S.stw, ar, 1, sload, [] {}, gstore);
     }
 }
 
 // Per-limb modular tables, in device memory (built on the host once per
 // context; the tables follow the array of these).
 struct NttLimb {
-    const ulonglong2 *fwd;   // [N]: (psi^brv(k), Shoup companion)
-    const ulonglong2 *inv;   // [N]: (psi^-brv(k), Shoup companion)
-    const ulonglong2 *qinv;  // [L]: q_j^-1 mod q (Shoup) for j > this limb, else (0, 0)
+    TwiddleTable fwd;        // [N]: psi^brv(k)
+    TwiddleTable inv;        // [N]: psi^-brv(k)
+    const Twiddle *qinv;     // [L]: q_j^-1 mod q for j > this limb, else 0
     uint64_t q;
     uint64_t mu64;           // floor(2^64 / q)
-    ulonglong2 ninv;         // N^-1 mod q (Shoup)
+    Twiddle ninv;            // N^-1 mod q
 };
 
 // host: log2 of a power of two

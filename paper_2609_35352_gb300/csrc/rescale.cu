@@ -20,6 +20,14 @@
 // last limb must be known before any limb can be finished, so the rescale
 // cannot share a launch with the layer's kernels, whose CTAs each see one
 // tile of coefficients.
+//
+// What bounds it: the FMA-heavy pipe (64-bit products, 4 cycles a warp), which
+// ncu shows 76% busy in the forward high pass and 62% in the low one, whose
+// epilogue also reads y.  Measured on GB300 (192 polys of 2^16, 12 -> 11
+// limbs): 1.728 ms with Shoup's product and one poly a low-pass CTA, 1.636 ms
+// with the two-word twiddles of ntt.cuh and four polys, 1.488 ms with their
+// tables in staging order (and N^-1, q^-1 in the same form), 1.410 ms with
+// eight polys; its HBM bytes take 0.34 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,49 +47,56 @@ struct Args {
     uint64_t *polys;   // [count][Lc][N]
     uint64_t *out;     // [count][Lc-1][N]
     const NttLimb *T;
+    uint32_t count;
     uint32_t Lc;
     uint32_t round;    // 1: nearest quotient (add h = floor(q_{Lc-1} / 2))
 };
 
 // ---------------------------------------------------------------------------
 // The four launches.  blockIdx.x = transform * tiles + tile; the transforms
-// are the polys (inverse passes) or poly * (Lc - 1) + limb (forward passes).
+// are the polys (inverse high pass), poly * (Lc - 1) + limb (forward high
+// pass), and for the low passes, whose CTAs take the same rows of kPolys
+// polys, group of polys (inverse) or group * (Lc - 1) + limb (forward).
 // ---------------------------------------------------------------------------
 
 // inverse, low stages, on the last limb in place
 template <int LOGN>
-__global__ void __launch_bounds__(LowPass<LOGN>::threads, 4) k_inv_low(Args A)
+__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 3) k_inv_low(Args A)
 {
-    using SH = Shape<LOGN>;
-    using PS = LowPass<LOGN>;
+    using PS = LowPassPolys<LOGN>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p = blockIdx.x >> PS::ltiles;
-    const uint32_t first = tile << PS::lsubs;
-    uint64_t *g = A.polys + ((size_t)p * A.Lc + (A.Lc - 1)) * (1u << LOGN) + ((size_t)first << PS::s);
+    const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p0 = (blockIdx.x >> PS::ltiles) << PS::lpolys;
+    const uint32_t first = tile << PS::lrows;
+    const size_t stride = (size_t)A.Lc << LOGN;
+    uint64_t *g = A.polys + p0 * stride + ((size_t)(A.Lc - 1) << LOGN) + ((size_t)first << PS::s);
     const NttLimb &Tl = A.T[A.Lc - 1];
-    inv_low_pass<LOGN>(smem_raw, Tl.inv, first, ModArith<false>{Tl.q}, [&](uint32_t e) { return g[e]; },
-                       [&](uint32_t sub, uint32_t pos, uint64_t v) { g[(sub << PS::s) + pos] = v; });
+    constexpr int le = PS::s + PS::lrows;  // log2 elements per poly
+    inv_low_pass<LOGN, PS>(
+        smem_raw, Tl.inv, first, ModArith<false>{Tl.q}, A.count - p0,
+        [&](uint32_t e0, uint32_t t) { return g[(e0 >> le) * stride + (e0 & ((1u << le) - 1)) + t]; },
+        [&](uint32_t sub, uint32_t pos, uint64_t v) {
+            g[(sub >> PS::lrows) * stride + ((sub & (PS::rows - 1)) << PS::s) + pos] = v;
+        });
 }
 
 // inverse, high stages: stores r = N^-1 x, canonical
 template <int LOGN>
 __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_inv_high(Args A)
 {
-    using SH = Shape<LOGN>;
     using PS = HighPass<LOGN>;
-    constexpr uint32_t R2 = 1u << (LOGN - SH::n1);
+    constexpr uint32_t R2 = 1u << (LOGN - Shape<LOGN>::n1);
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p = blockIdx.x >> PS::ltiles;
     const uint32_t first = tile << PS::lsubs;
     uint64_t *g = A.polys + ((size_t)p * A.Lc + (A.Lc - 1)) * (1u << LOGN) + first;
     const NttLimb &Tl = A.T[A.Lc - 1];
     const uint64_t q = Tl.q;
-    const ulonglong2 ninv = Tl.ninv;
+    const Twiddle ninv = Tl.ninv;
     const uint64_t h = A.round ? q / 2 : 0;
     inv_high_pass<LOGN>(smem_raw, Tl.inv, first, ModArith<false>{q},
                         [&](uint32_t sub, uint32_t pos) { return g[(size_t)pos * R2 + sub]; },
                         [&](uint32_t sub, uint32_t pos, uint64_t v) {
-                            g[(size_t)pos * R2 + sub] = csub(canon4(mul_shoup_lazy(v, ninv, q), q) + h, q);
+                            g[(size_t)pos * R2 + sub] = csub(canon6(mul_twiddle(v, ninv, q), q) + h, q);
                         });
 }
 
@@ -90,9 +105,8 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_inv_high(Args A)
 template <int LOGN, bool FAST>
 __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_fwd_high(Args A)
 {
-    using SH = Shape<LOGN>;
     using PS = HighPass<LOGN>;
-    constexpr uint32_t R2 = 1u << (LOGN - SH::n1);
+    constexpr uint32_t R2 = 1u << (LOGN - Shape<LOGN>::n1);
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), tr = blockIdx.x >> PS::ltiles;
     const uint32_t p = tr / (A.Lc - 1), l = tr % (A.Lc - 1);
@@ -115,32 +129,42 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_fwd_high(Args A)
 
 // forward, low stages, then y' = (y_l - t) * q_{Lc-1}^-1
 template <int LOGN, bool FAST>
-__global__ void __launch_bounds__(LowPass<LOGN>::threads, 4) k_fwd_low(Args A)
+__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 3) k_fwd_low(Args A)
 {
-    using SH = Shape<LOGN>;
-    using PS = LowPass<LOGN>;
+    using PS = LowPassPolys<LOGN>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), tr = blockIdx.x >> PS::ltiles;
-    const uint32_t p = tr / (A.Lc - 1), l = tr % (A.Lc - 1);
-    const uint32_t first = tile << PS::lsubs;
-    uint64_t *o = A.out + (size_t)tr * (1u << LOGN) + ((size_t)first << PS::s);
-    const uint64_t *y = A.polys + ((size_t)p * A.Lc + l) * (1u << LOGN) + ((size_t)first << PS::s);
+    const uint32_t p0 = (tr / (A.Lc - 1)) << PS::lpolys, l = tr % (A.Lc - 1);
+    const uint32_t first = tile << PS::lrows;
+    const size_t so = (size_t)(A.Lc - 1) << LOGN, sy = (size_t)A.Lc << LOGN;
+    const size_t at = ((size_t)l << LOGN) + ((size_t)first << PS::s);
+    uint64_t *o = A.out + p0 * so + at;
+    const uint64_t *y = A.polys + p0 * sy + at;
+    const uint32_t np = A.count - p0;
     const NttLimb &Tl = A.T[l];
     const uint64_t q = Tl.q;
-    const ulonglong2 qi = Tl.qinv[A.Lc - 1];
-    // transform values: below 73q (FAST) or 8q; M = 128q or 8q bounds them
-    const uint64_t M = (FAST ? 128 : 8) * q;
-    fwd_low_pass<LOGN>(
-        smem_raw, Tl.fwd, first, ModArith<FAST>{q},
+    const Twiddle qi = Tl.qinv[A.Lc - 1];
+    // transform values: below 110q (FAST) or 12q; M = 128q or 12q bounds them
+    const uint64_t M = (FAST ? 128 : 12) * q;
+    constexpr int le = PS::s + PS::lrows;  // log2 elements per poly
+    fwd_low_pass<LOGN, PS>(
+        smem_raw, Tl.fwd, first, ModArith<FAST>{q}, np,
         [&] {
             // y is read only by the epilogue: start bringing it into L2 now
             for (uint32_t e = threadIdx.x * 16; e < PS::tile; e += PS::threads * 16)
-                asm volatile("prefetch.global.L2 [%0];\n" ::"l"(y + e));
+                if ((e >> le) < np)
+                    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(y + (e >> le) * sy + (e & ((1u << le) - 1))));
         },
-        [&](uint32_t sub, uint32_t pos) { return o[(sub << PS::s) + pos]; },
+        [&](uint32_t sub, uint32_t pos) {
+            return o[(sub >> PS::lrows) * so + ((sub & (PS::rows - 1)) << PS::s) + pos];
+        },
         [&](auto t_of) {
-            sweep<PS, uint64_t>([&](uint32_t e) { return y[e]; },
-                                [&](uint32_t e, uint64_t v) { o[e] = canon4(mul_shoup_lazy(v + M - t_of(e), qi, q), q); });
+            sweep<PS, uint64_t>(
+                np, [&](uint32_t e0, uint32_t t) { return y[(e0 >> le) * sy + (e0 & ((1u << le) - 1)) + t]; },
+                [&](uint32_t e0, uint32_t t, uint64_t v) {
+                    o[(e0 >> le) * so + (e0 & ((1u << le) - 1)) + t] =
+                        canon6(mul_twiddle(v + M - t_of(e0, t), qi, q), q);
+                });
         });
 }
 
@@ -160,7 +184,16 @@ uint64_t powm(uint64_t b, uint64_t e, uint64_t q)
     return r;
 }
 
-ulonglong2 shoup(uint64_t w, uint64_t q) { return make_ulonglong2(w, (uint64_t)(((u128)w << 64) / q)); }
+// the table entry of w (ntt.cuh): 2^32 w mod q, and both quotients by 2q
+Twiddle twiddle(uint64_t w, uint64_t q)
+{
+    const u128 w32 = (u128)w << 32;
+    const uint64_t qw = (uint64_t)(w32 / q), v = (uint64_t)w32 - qw * q;
+    Twiddle t;
+    t.wv = make_ulonglong2(w, v);
+    t.om = make_uint2((uint32_t)(qw / 2), (uint32_t)(((u128)v << 31) / q));
+    return t;
+}
 
 // The least primitive 2N-th root of unity mod q, or 0.  For the first x whose
 // c = x^((q-1)/2N) has c^N = -1, c is primitive and the primitive roots are
@@ -194,9 +227,11 @@ int build_tables(const fiona_ctx *ctx)
     std::lock_guard<std::mutex> lock(g_ntt_mu);
     if (ctx->d_ntt) return FIONA_OK;
     const uint32_t N = ctx->N, L = ctx->L;
-    const uint32_t n = log2u(N);
+    // the shape of the low pass (LowPassPolys): n1 stages in the high pass,
+    // tiles of 2^lrows rows
+    const uint32_t n = log2u(N), n1 = n / 2, lrows = kLogTileMax - (n - n1) - kLogPolys;
     const size_t head = ((sizeof(NttLimb) * L + 255) / 256) * 256;
-    const size_t table = sizeof(ulonglong2) * N, qtab = sizeof(ulonglong2) * L;
+    const size_t wv = sizeof(ulonglong2) * N, om = sizeof(uint2) * N, table = wv + om, qtab = sizeof(Twiddle) * L;
     const size_t per_limb = 2 * table + ((qtab + 255) / 256) * 256;
     const size_t bytes = head + per_limb * L;
     std::vector<uint8_t> host(bytes, 0);
@@ -212,26 +247,32 @@ int build_tables(const fiona_ctx *ctx)
             return set_error(FIONA_ERR_MODULUS, "rescale: modulus %u has no primitive 2N-th root of unity", l);
         }
         const size_t off = head + per_limb * l;
-        ulonglong2 *fwd = reinterpret_cast<ulonglong2 *>(host.data() + off);
-        ulonglong2 *inv = reinterpret_cast<ulonglong2 *>(host.data() + off + table);
-        ulonglong2 *qinv = reinterpret_cast<ulonglong2 *>(host.data() + off + 2 * table);
+        Twiddle *qinv = reinterpret_cast<Twiddle *>(host.data() + off + 2 * table);
         // powers of psi, then of psi^-1, placed in bit-reversed order
         for (int dir = 0; dir < 2; ++dir) {
             const uint64_t base = dir == 0 ? psi : powm(psi, q - 2, q);
             pw[0] = 1;
             for (uint32_t i = 1; i < N; ++i) pw[i] = mulm(pw[i - 1], base, q);
-            ulonglong2 *dst = dir == 0 ? fwd : inv;
-            for (uint32_t k = 0; k < N; ++k) dst[k] = shoup(pw[bit_reverse(k, n)], q);
+            ulonglong2 *d_wv = reinterpret_cast<ulonglong2 *>(host.data() + off + dir * table);
+            uint2 *d_om = reinterpret_cast<uint2 *>(host.data() + off + dir * table + wv);
+            for (uint32_t k = 0; k < N; ++k) {
+                const Twiddle t = twiddle(pw[bit_reverse(k, n)], q);
+                const uint32_t at = low_place(k, n1, n - n1, lrows);
+                d_wv[at] = t.wv;
+                d_om[at] = t.om;
+            }
         }
-        for (uint32_t j = l + 1; j < L; ++j) qinv[j] = shoup(powm(ctx->moduli[j] % q, q - 2, q), q);
+        for (uint32_t j = l + 1; j < L; ++j) qinv[j] = twiddle(powm(ctx->moduli[j] % q, q - 2, q), q);
         NttLimb &T = reinterpret_cast<NttLimb *>(host.data())[l];
         const uint8_t *dbase = static_cast<const uint8_t *>(dev) + off;
-        T.fwd = reinterpret_cast<const ulonglong2 *>(dbase);
-        T.inv = reinterpret_cast<const ulonglong2 *>(dbase + table);
-        T.qinv = reinterpret_cast<const ulonglong2 *>(dbase + 2 * table);
+        T.fwd.wv = reinterpret_cast<const ulonglong2 *>(dbase);
+        T.fwd.om = reinterpret_cast<const uint2 *>(dbase + wv);
+        T.inv.wv = reinterpret_cast<const ulonglong2 *>(dbase + table);
+        T.inv.om = reinterpret_cast<const uint2 *>(dbase + table + wv);
+        T.qinv = reinterpret_cast<const Twiddle *>(dbase + 2 * table);
         T.q = q;
         T.mu64 = ~(uint64_t)0 / q;
-        T.ninv = shoup(powm(N % q, q - 2, q), q);
+        T.ninv = twiddle(powm(N % q, q - 2, q), q);
     }
     e = cudaMemcpy(dev, host.data(), bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -285,17 +326,17 @@ int launch_rescale(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64_t cou
     // per pass: tiles per transform (log2) and threads per CTA
 #define FIONA_GEO(P) {P<10>::ltiles, P<11>::ltiles, P<12>::ltiles, P<13>::ltiles, P<14>::ltiles, P<15>::ltiles, P<16>::ltiles, P<17>::ltiles}
 #define FIONA_THR(P) {P<10>::threads, P<11>::threads, P<12>::threads, P<13>::threads, P<14>::threads, P<15>::threads, P<16>::threads, P<17>::threads}
-    static const int low_lt[] = FIONA_GEO(LowPass), high_lt[] = FIONA_GEO(HighPass);
-    static const uint32_t low_thr[] = FIONA_THR(LowPass), high_thr[] = FIONA_THR(HighPass);
+    static const int low_lt[] = FIONA_GEO(LowPassPolys), high_lt[] = FIONA_GEO(HighPass);
+    static const uint32_t low_thr[] = FIONA_THR(LowPassPolys), high_thr[] = FIONA_THR(HighPass);
 #undef FIONA_GEO
 #undef FIONA_THR
     const uint32_t lt_low = (uint32_t)low_lt[ix], lt_high = (uint32_t)high_lt[ix];
     const Kern ks[4] = {inv_low[ix], inv_high[ix], fwd_high[fast][ix], fwd_low[fast][ix]};
     typedef ModArith<false> MA;
     static const size_t low_smem[] = {
-        LowPass<10>::smem_bytes<MA>(), LowPass<11>::smem_bytes<MA>(), LowPass<12>::smem_bytes<MA>(),
-        LowPass<13>::smem_bytes<MA>(), LowPass<14>::smem_bytes<MA>(), LowPass<15>::smem_bytes<MA>(),
-        LowPass<16>::smem_bytes<MA>(), LowPass<17>::smem_bytes<MA>()};
+        LowPassPolys<10>::smem_bytes<MA>(), LowPassPolys<11>::smem_bytes<MA>(), LowPassPolys<12>::smem_bytes<MA>(),
+        LowPassPolys<13>::smem_bytes<MA>(), LowPassPolys<14>::smem_bytes<MA>(), LowPassPolys<15>::smem_bytes<MA>(),
+        LowPassPolys<16>::smem_bytes<MA>(), LowPassPolys<17>::smem_bytes<MA>()};
     static const size_t high_smem[] = {
         HighPass<10>::smem_bytes<MA>(), HighPass<11>::smem_bytes<MA>(), HighPass<12>::smem_bytes<MA>(),
         HighPass<13>::smem_bytes<MA>(), HighPass<14>::smem_bytes<MA>(), HighPass<15>::smem_bytes<MA>(),
@@ -326,13 +367,14 @@ int launch_rescale(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64_t cou
         a.polys = polys + p0 * Lc * (uint64_t)ctx->N;
         a.out = out + p0 * (Lc - 1) * (uint64_t)ctx->N;
         a.T = T;
+        a.count = (uint32_t)np;
         a.Lc = Lc;
         a.round = round ? 1 : 0;
-        const uint64_t nf = np * (Lc - 1);
-        ks[0]<<<(uint32_t)(np << lt_low), low_thr[ix], smem[0], s>>>(a);
+        const uint64_t nf = np * (Lc - 1), ng = (np + kPolys - 1) / kPolys;
+        ks[0]<<<(uint32_t)(ng << lt_low), low_thr[ix], smem[0], s>>>(a);
         ks[1]<<<(uint32_t)(np << lt_high), high_thr[ix], smem[1], s>>>(a);
         ks[2]<<<(uint32_t)(nf << lt_high), high_thr[ix], smem[2], s>>>(a);
-        ks[3]<<<(uint32_t)(nf << lt_low), low_thr[ix], smem[3], s>>>(a);
+        ks[3]<<<(uint32_t)((ng * (Lc - 1)) << lt_low), low_thr[ix], smem[3], s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "rescale launch: %s", cudaGetErrorString(e));
