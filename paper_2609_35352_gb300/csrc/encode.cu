@@ -136,6 +136,11 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_enc_high(EncArgs
         smem_raw, Tl.fwd, first, ModArith<FAST>{q},
         [&](uint32_t sub, uint32_t pos) {
             const int64_t v = c[(size_t)pos * R2 + sub];
+            // the coefficients of a plaintext are mostly far below q: v + 4q
+            // is then a value the reduction-free butterflies take, for two
+            // additions and a comparison in place of a 64-bit high product
+            // (GB300, 93 plaintexts of 2^16 at 12 limbs: 0.685 -> 0.631 ms)
+            if (FAST && (uint64_t)v + 4 * q < 8 * q) return (uint64_t)v + 4 * q;
             // |v| as an unsigned word (exact for every 64-bit v); -|v| is q - r,
             // in (0, q]
             const uint64_t mag = v >= 0 ? (uint64_t)v : 0 - (uint64_t)v;
