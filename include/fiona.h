@@ -78,7 +78,10 @@ typedef enum fiona_status {
  * into shared memory (bulk asynchronous copies), shared signed sums are
  * formed once per tile, and the warps split the outputs.  AUTO (the default
  * after fiona_plan_create): TILED for layers with more than one output whose
- * tile fits in shared memory, DIRECT otherwise. */
+ * tile fits in shared memory, DIRECT otherwise.  For a layer whose every raw
+ * plaintext is constant, TILED is the matrix kernel where the layer is large
+ * enough for it (tile_coeffs 128: 128 coefficients of one poly per CTA, both
+ * routes as exact products on the tensor cores). */
 enum { FIONA_KERNEL_AUTO = 0, FIONA_KERNEL_DIRECT = 1, FIONA_KERNEL_TILED = 2 };
 
 /* Pass as `device` to fiona_ctx_create for a validation-only context: plans
@@ -168,7 +171,8 @@ typedef struct fiona_plan_stats_t {
                                      an output's products, its partial sums) counts n - 1 */
     uint32_t tensor_core_sums;    /* TILED: scale-group signed sums formed per tile as one
                                      contraction on the tensor cores (the groups' terms, shared
-                                     sums expanded, exact in fp16 chunks); 0: on the ALUs      */
+                                     sums expanded, exact in fp16 chunks; always with the matrix
+                                     kernel); 0: on the ALUs                                  */
     uint32_t source_offsets;      /* TILED: 1 if the schedule's signed-sum runs hold source byte
                                      offsets (one addition per source address), 0 if 16-bit
                                      indices packed two per word (used when the larger offset

@@ -32,8 +32,8 @@ EXTRA = {"kernel_tiled.cu": ["-Xptxas", "-regUsageLevel=8"],
          "kernel_tiled_w12.cu": ["-Xptxas", "-regUsageLevel=8"]}
 
 LIBRARIES = {
-    "libfiona.so": ["fiona_host.cpp", "lower_tiled.cpp", "plan_compile.cpp", "kernel_direct.cu",
-                    "kernel_tiled.cu", "kernel_tiled_off.cu", "kernel_tiled_w12.cu", "kernel_ws.cu", "rescale.cu", "encode.cu"],
+    "libfiona.so": ["fiona_host.cpp", "lower_tiled.cpp", "lower_gemm.cpp", "plan_compile.cpp", "kernel_direct.cu",
+                    "kernel_tiled.cu", "kernel_tiled_off.cu", "kernel_tiled_w12.cu", "kernel_ws.cu", "kernel_gemm.cu", "rescale.cu", "encode.cu"],
     "libfiona_workload.so": ["workload_fill.cu", "mul_roof.cu"],
 }
 

@@ -11,6 +11,7 @@
 #include <new>
 
 #include "fiona_internal.h"
+#include "gemm.h"
 #include "tiled.h"
 
 typedef unsigned __int128 u128;
@@ -527,11 +528,13 @@ static void build_static_image(fiona_plan *p)
 static void release_device(fiona_plan *p)
 {
     if (!p->ctx || p->ctx->device == FIONA_DEVICE_NONE) {
-        if (p->tiled) free_tiled(p);  // host-only schedule: nothing on a device
+        if (p->tiled) free_tiled(p);  // host-only schedules: nothing on a device
+        free_gemm(p);
         return;
     }
     DeviceGuard g(p->ctx->device);
     if (p->tiled) free_tiled(p);
+    free_gemm(p);
     cudaFree(p->sched.blob);
     p->sched.blob = nullptr;
     if (p->copy_in_stream) cudaStreamDestroy((cudaStream_t)p->copy_in_stream);
@@ -555,8 +558,15 @@ static int lower_tiled_optional(fiona_plan *p)
     const int rc = lower_tiled(p);
     if (rc == FIONA_ERR_INTERNAL) return rc;
     if (rc != FIONA_OK) p->tiled = nullptr;
+    if (p->tiled && lower_gemm(p) != FIONA_OK) free_gemm(p);
     set_error(FIONA_OK, "");
     return FIONA_OK;
+}
+
+// Whether a launch of `n_limbs` limbs takes the matrix kernel
+static bool use_gemm(const fiona_plan *p, uint32_t n_limbs)
+{
+    return p->kernel == 1 && p->gemm && gemm_units(p, n_limbs) >= p->gemm->min_units;
 }
 
 // Kernel choice: TILED for layers with more than one output whose tile fits
@@ -577,7 +587,18 @@ static int select_kernel(fiona_plan *p, int which)
         return set_error(FIONA_ERR_ARG, "select_kernel: the tiled kernel cannot run this plan");
     p->kernel = k;
     fiona_plan_stats_t &s = p->stats;
-    if (k == 1 && p->tiled) {
+    if (use_gemm(p, p->ctx->L)) {
+        s.kernel = FIONA_KERNEL_TILED;
+        s.tile_coeffs = kGemmRows;
+        s.warps_per_cta = kGemmThreads / 32;
+        s.smem_bytes = (uint32_t)p->gemm->smem;
+        s.ctas_per_sm = 1;
+        s.nodes_materialized = 0;
+        s.addsub_executed = (uint32_t)std::min<uint64_t>(s.addsub_flat, 0xffffffffu);
+        s.tensor_core_sums = p->gemm->groups;
+        s.source_offsets = 0;
+        s.const_raw_all = 1;
+    } else if (k == 1 && p->tiled) {
         s.kernel = FIONA_KERNEL_TILED;
         s.tile_coeffs = p->tiled->tile;
         s.warps_per_cta = p->tiled->warps;
@@ -819,6 +840,7 @@ static int check_eval_args(const fiona_plan *p, const void *in, const void *pt, 
 static int launch_range(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt,
                         uint64_t *out, uint32_t l0, uint32_t l1, uint32_t layout_L)
 {
+    if (use_gemm(p, l1 - l0)) return launch_gemm(p, stream, in, pt, out, l0, l1, layout_L);
     if (p->kernel == 1) return launch_tiled(p, stream, in, pt, out, l0, l1, layout_L);
     return launch_direct(p, stream, in, pt, out, l0, l1, layout_L);
 }

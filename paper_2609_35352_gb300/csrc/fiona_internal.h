@@ -33,6 +33,7 @@ struct DirSeg {
 // warp owns a job list).  Defined in lower_tiled.cpp / kernel_tiled.cu.
 // ---------------------------------------------------------------------------
 struct TiledSchedule;
+struct GemmSchedule;  // gemm.h: the matrix kernel for layers with constant raw plaintexts
 
 struct DeviceSchedule {
     void *blob = nullptr;  // one device allocation holding every array below
@@ -83,6 +84,9 @@ struct fiona_plan {
     const uint32_t *d_raw_pt = nullptr;
     // tiled schedule
     TiledSchedule *tiled = nullptr;
+    // matrix kernel's schedule, where it can run the layer and pays: the
+    // tiled variant of such a plan for launches of enough units
+    GemmSchedule *gemm = nullptr;
     // streams for fiona_linear_eval_host(_async), and per limb chunk the
     // events of its last input copy, kernel and output copy: a call orders
     // each chunk after the previous call's use of the same device buffers
@@ -115,6 +119,14 @@ int lower_tiled(fiona_plan *p);
 void free_tiled(fiona_plan *p);
 int launch_tiled(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt,
                  uint64_t *out, uint32_t limb_begin, uint32_t limb_end, uint32_t layout_L);
+
+// lower_gemm.cpp / kernel_gemm.cu (optional: p->gemm stays null where it does
+// not apply)
+int lower_gemm(fiona_plan *p);
+void free_gemm(fiona_plan *p);
+uint32_t gemm_units(const fiona_plan *p, uint32_t n_limbs);
+int launch_gemm(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt, uint64_t *out,
+                uint32_t limb_begin, uint32_t limb_end, uint32_t layout_L);
 
 // rescale.cu.  Rescales `count` polys [count][Lc][N] (the last limb of each
 // is overwritten with its coefficients) into out [count][Lc-1][N].
