@@ -83,10 +83,10 @@ direct_kernel(const uint64_t *__restrict__ in, const uint64_t *__restrict__ pt,
             }
         }
         const ulonglong2 g = ld2(ptl + (size_t)sg.scale_pt * LN);
-        rns::mac(lo[0][0], hi[0][0], g.x, S[0][0]);
-        rns::mac(lo[0][1], hi[0][1], g.y, S[0][1]);
-        rns::mac(lo[1][0], hi[1][0], g.x, S[1][0]);
-        rns::mac(lo[1][1], hi[1][1], g.y, S[1][1]);
+        rns::mac128(lo[0][0], hi[0][0], g.x, S[0][0]);
+        rns::mac128(lo[0][1], hi[0][1], g.y, S[0][1]);
+        rns::mac128(lo[1][0], hi[1][0], g.x, S[1][0]);
+        rns::mac128(lo[1][1], hi[1][1], g.y, S[1][1]);
         fold_if_full();
     }
 #pragma unroll 2
@@ -98,10 +98,10 @@ direct_kernel(const uint64_t *__restrict__ in, const uint64_t *__restrict__ pt,
         if (wp >> 31) p.y = p.x;
         const ulonglong2 a0 = ld2(inl + (size_t)(2 * i) * LN);
         const ulonglong2 a1 = ld2(inl + (size_t)(2 * i + 1) * LN);
-        rns::mac(lo[0][0], hi[0][0], p.x, a0.x);
-        rns::mac(lo[0][1], hi[0][1], p.y, a0.y);
-        rns::mac(lo[1][0], hi[1][0], p.x, a1.x);
-        rns::mac(lo[1][1], hi[1][1], p.y, a1.y);
+        rns::mac128(lo[0][0], hi[0][0], p.x, a0.x);
+        rns::mac128(lo[0][1], hi[0][1], p.y, a0.y);
+        rns::mac128(lo[1][0], hi[1][0], p.x, a1.x);
+        rns::mac128(lo[1][1], hi[1][1], p.y, a1.y);
         fold_if_full();
     }
     uint64_t *outl = out + ((size_t)j * 2 * L + l) * N + k;

@@ -321,6 +321,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
                     A::mac(acc[0][x], gg, s0.x[x]);
                     A::mac(acc[1][x], gg, s1.x[x]);
                 }
+                if ((i + 1) % rns::kMidBudget == 0 || i + 1 == P) settle_all<A, C>(acc);
             }
             if (++slot == D) slot = 0;
             if (hw[P - 1] & kOpLast) finish();

@@ -8,7 +8,8 @@
 //   narrow: rns::mac26, three 32x32 -> 64-bit products of radix-2^26 halves
 //           (Karatsuba) into three accumulators -- one 50-bit x 50-bit
 //           product per call;
-//   wide:   rns::mac, the 64x64 -> 128-bit product-accumulate with carry.
+//   wide:   rns::mac, the 60-bit product-accumulate in 32-bit halves, settled
+//           every rns::kMidBudget steps.
 // The rate is products per second of the whole GPU, timed with CUDA events
 // after a warm-up launch.  A layer's products per evaluation
 // (fiona_plan_stats.wide_products) over its kernel time, divided by this
@@ -41,7 +42,8 @@ __global__ void __launch_bounds__(256) roof_kernel(const uint64_t *seed, uint64_
             if (NARROW)
                 rns::mac26(lo[c], mid[c], hi[c], a[c], b[c], zero);  // as the layer kernels call it
             else
-                rns::mac(lo[c], hi[c], a[c], b[c]);
+                rns::mac(lo[c], mid[c], hi[c], a[c], b[c]);
+            if (!NARROW && s % rns::kMidBudget == rns::kMidBudget - 1) rns::settle(lo[c], mid[c], hi[c]);
             // the next step's operands depend on this step (stay in split form)
             a[c] = (a[c] + (lo[c] & 0x0000000F0000000Full)) & 0x03FFFFFF03FFFFFFull;
         }

@@ -44,8 +44,51 @@ struct LimbConst {
 #if defined(__CUDACC__)
 namespace rns {
 
-// acc (lo, hi) += a * b, full 128-bit product, carry chained.
-__device__ __forceinline__ void mac(uint64_t &lo, uint64_t &hi, uint64_t a, uint64_t b)
+// (lo, hi) + mid 2^32 += a * b for residues a, b < 2^60, in 32-bit halves: the
+// low and the high product are one carry chain, the two middle products (each
+// below 2^60) add into a word of their own, which holds kMidBudget of them:
+// settle() moves it into (lo, hi).  Four multiply-adds a product; the chained
+// 64-bit form (mad.lo.cc.u64, madc.hi.u64) took the FMA-heavy pipe for 32 cycles
+// a product, warp and scheduler on GB300 against 21 here (register-only loop
+// with operands from shared memory).
+constexpr uint32_t kMidBudget = 8;
+
+__device__ __forceinline__ void mac(uint64_t &lo, uint64_t &mid, uint64_t &hi, uint64_t a, uint64_t b)
+{
+    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), b0 = (uint32_t)b, b1 = (uint32_t)(b >> 32);
+    uint32_t l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
+    asm("mad.lo.cc.u32  %0, %4, %6, %0;\n\t"
+        "madc.hi.cc.u32 %1, %4, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %7, %2;\n\t"
+        "madc.hi.u32    %3, %5, %7, %3;"
+        : "+r"(l0), "+r"(l1), "+r"(h0), "+r"(h1)
+        : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
+    lo = ((uint64_t)l1 << 32) | l0;
+    hi = ((uint64_t)h1 << 32) | h0;
+    asm("mad.wide.u32 %0, %1, %2, %0;\n\t"
+        "mad.wide.u32 %0, %3, %4, %0;"
+        : "+l"(mid)
+        : "r"(a0), "r"(b1), "r"(a1), "r"(b0));
+}
+
+__device__ __forceinline__ void settle(uint64_t &lo, uint64_t &mid, uint64_t &hi)
+{
+    uint32_t l1 = (uint32_t)(lo >> 32), h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
+    asm("add.cc.u32  %0, %0, %3;\n\t"
+        "addc.cc.u32 %1, %1, %4;\n\t"
+        "addc.u32    %2, %2, 0;"
+        : "+r"(l1), "+r"(h0), "+r"(h1)
+        : "r"((uint32_t)mid), "r"((uint32_t)(mid >> 32)));
+    lo = ((uint64_t)l1 << 32) | (uint32_t)lo;
+    hi = ((uint64_t)h1 << 32) | h0;
+    mid = 0;
+}
+
+// acc (lo, hi) += a * b, full 128-bit product, carry chained (the direct kernel's
+// form: it waits for memory, and the middle words of mac() below cost it more
+// registers than the multiplications save: the 64-ciphertext sum 0.338 ms
+// against 0.310 on GB300)
+__device__ __forceinline__ void mac128(uint64_t &lo, uint64_t &hi, uint64_t a, uint64_t b)
 {
     asm("mad.lo.cc.u64 %0, %2, %3, %0;\n\t"
         "madc.hi.u64   %1, %2, %3, %1;"

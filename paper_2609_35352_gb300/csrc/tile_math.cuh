@@ -82,15 +82,21 @@ __device__ __forceinline__ void stg(uint64_t *p, const V<C> &v)
 template <bool NARROW>
 struct Arith;
 
-// Any q < 2^60: 128-bit products (lo, hi), plain 64-bit sums.
+// Any q < 2^60: 128-bit products (lo, hi) with their middle parts apart until
+// settle() (at least every rns::kMidBudget products), plain 64-bit sums.
 template <>
 struct Arith<false> {
     struct Acc {
-        uint64_t lo, hi;
+        uint64_t lo, mid, hi;
     };
     __device__ static uint64_t operand(uint64_t a) { return a; }
-    __device__ static void zero(Acc &a) { a.lo = a.hi = 0; }
-    __device__ static void mac(Acc &a, uint64_t x, uint64_t y, uint32_t /*zero*/ = 0) { rns::mac(a.lo, a.hi, x, y); }
+    __device__ static void zero(Acc &a) { a.lo = a.mid = a.hi = 0; }
+    __device__ static void mac(Acc &a, uint64_t x, uint64_t y, uint32_t /*zero*/ = 0)
+    {
+        rns::mac(a.lo, a.mid, a.hi, x, y);
+    }
+    __device__ static void settle(Acc &a) { rns::settle(a.lo, a.mid, a.hi); }
+    // (a settled accumulator)
     __device__ static uint64_t reduce(const Acc &a, const LimbConst &m) { return rns::reduce128(a.lo, a.hi, m); }
     __device__ static void fold(Acc &a, const LimbConst &m)
     {
@@ -127,6 +133,7 @@ struct Arith<true> {
     {
         rns::mac26(a.lo, a.x, a.hi, x, y, zero);
     }
+    __device__ static void settle(Acc &) {}
     __device__ static uint64_t reduce(const Acc &a, const LimbConst &m) { return rns::reduce26(a.lo, a.x, a.hi, m); }
     __device__ static void fold(Acc &a, const LimbConst &m)
     {
@@ -141,6 +148,16 @@ struct Arith<true> {
         return rns::reduce64(rns::unsplit_sum(p) + k - rns::unsplit_sum(mm), m);
     }
 };
+
+// the accumulators of both polys, settled (nothing for narrow moduli)
+template <class A, int C>
+__device__ __forceinline__ void settle_all(typename A::Acc (&acc)[2][C])
+{
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int x = 0; x < C; ++x) A::settle(acc[c][x]);
+}
 
 // Sum of the n source tiles (both polys) named by the 16-bit indices packed
 // two per word from schedule byte offset `wp`; `src` = this lane's offset in

@@ -577,6 +577,7 @@ __global__ void __launch_bounds__(WB * 32)
                     A::mac(acc[0][x], g, s0.x[x], zero);
                     A::mac(acc[1][x], g, s1.x[x], zero);
                 }
+                if ((i + 1) % rns::kMidBudget == 0 || i + 1 == P) settle_all<A, C>(acc);
                 r[i] = fetch(nb, nlb, ns, nwi, i);
             }
             if (cw4.w & kOpLast) finish();  // the batch's last word
