@@ -78,7 +78,8 @@ typedef enum fiona_status {
  * into shared memory (bulk asynchronous copies), shared signed sums are
  * formed once per tile, and the warps split the outputs.  AUTO (the default
  * after fiona_plan_create): TILED for layers with more than one output whose
- * tile fits in shared memory, DIRECT otherwise.  For a layer whose every raw
+ * tile fits in shared memory and whose outputs read more than a few operands,
+ * DIRECT otherwise.  For a layer whose every raw
  * plaintext is constant, TILED is the matrix kernel where the layer is large
  * enough for it (tile_coeffs 128: 128 coefficients of one poly per CTA, both
  * routes as exact products on the tensor cores). */

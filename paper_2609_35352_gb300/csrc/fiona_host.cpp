@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <new>
@@ -555,6 +556,7 @@ static void release_device(fiona_plan *p)
 // a library bug and is reported.
 static int lower_tiled_optional(fiona_plan *p)
 {
+    p->shape_asked = getenv("FIONA_TILED_SHAPE") || getenv("FIONA_TILED_TC") || getenv("FIONA_TILED_WS");
     const int rc = lower_tiled(p);
     if (rc == FIONA_ERR_INTERNAL) return rc;
     if (rc != FIONA_OK) p->tiled = nullptr;
@@ -569,9 +571,31 @@ static bool use_gemm(const fiona_plan *p, uint32_t n_limbs)
     return p->kernel == 1 && p->gemm && gemm_units(p, n_limbs) >= p->gemm->min_units;
 }
 
-// Kernel choice: TILED for layers with more than one output whose tile fits
-// in shared memory (every input is then read from HBM once), DIRECT otherwise
-// (a single output has no input reuse to exploit).
+// Layers whose outputs read few operands: the tiled kernel's tile (staging,
+// padded batches, one barrier) then costs more than the direct kernel's
+// repeated reads through L2.  Measured on GB300, tiled against direct time:
+// 3 -> 16 outputs 1.2-1.7, 4 -> 4 1.0-1.4, 6 -> 6 1.1-1.3 (N = 2^10 to 2^16, 2
+// to 24 limbs); the smallest layer, whose 16 scale groups of one term each open
+// a batch of their own, 10.2 us against 8.2; 60-bit moduli 8 -> 8 1.15 and 10 ->
+// 10 1.09 at 2^16 and 12 limbs (and 0.8 for 8 -> 4 at 2^12 and 3 limbs, hence
+// the size bound); 50-bit moduli 8 -> 8 1.0, 10 -> 10 0.92; two outputs of 8
+// operands 1.25-1.85.
+static bool few_operands(const fiona_plan *p)
+{
+    const fiona_plan_stats_t &s = p->stats;
+    const uint64_t terms = s.n_nonzero_terms, n_out = p->hp.n_out;
+    if (terms <= 6 * n_out) return true;
+    // operations once each scale group opens a batch of four
+    if (p->hp.n_in <= 8 && 4 * std::max<uint64_t>(s.n_scale_groups_used, n_out) >= 2 * terms) return true;
+    if ((uint64_t)p->ctx->N * p->ctx->L * n_out < (1u << 17)) return false;
+    const bool wide = p->ctx->q_max >= (1ull << 52);
+    return (wide && terms <= 10 * n_out) || (n_out <= 2 && terms <= 16 * n_out);
+}
+
+// Kernel choice: DIRECT for a single output (no input reuse to exploit), where
+// the tile does not fit in shared memory, and for layers of few operands an
+// output, unless a shape of the tiled kernel is asked for; TILED otherwise
+// (every input is then read from HBM once).
 static int select_kernel(fiona_plan *p, int which)
 {
     int k;
@@ -580,7 +604,7 @@ static int select_kernel(fiona_plan *p, int which)
     else if (which == FIONA_KERNEL_TILED)
         k = 1;
     else if (which == FIONA_KERNEL_AUTO)
-        k = (p->tiled && p->hp.n_out > 1) ? 1 : 0;
+        k = (p->tiled && p->hp.n_out > 1 && (p->shape_asked || p->gemm || !few_operands(p))) ? 1 : 0;
     else
         return set_error(FIONA_ERR_ARG, "select_kernel: unknown variant %d", which);
     if (k == 1 && !p->tiled && p->ctx->device != FIONA_DEVICE_NONE)

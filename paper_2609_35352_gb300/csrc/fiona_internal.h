@@ -75,6 +75,7 @@ struct fiona_plan {
     uint32_t mac_budget = 0;     // products a 128-bit accumulator may take before a reduction
     uint32_t signed_budget = 0;  // residues a 64-bit signed accumulator may take
     int kernel = 0;              // 0 = direct, 1 = tiled (what evaluations use)
+    bool shape_asked = false;    // a tuning override named a shape of the tiled kernel
     // direct schedule (device pointers into sched.blob)
     DeviceSchedule sched;
     const DirOut *d_dir_out = nullptr;

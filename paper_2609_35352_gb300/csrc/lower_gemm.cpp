@@ -37,8 +37,7 @@ int lower_gemm(fiona_plan *p)
     const char *env = getenv("FIONA_CONST_GEMM");
     const bool off = env && env[0] == '0', force = env && env[0] == '1';
     // a forced shape of the tiled kernel is a request for that kernel
-    if (off || (!force && (getenv("FIONA_TILED_SHAPE") || getenv("FIONA_TILED_TC") || getenv("FIONA_TILED_WS"))))
-        return FIONA_OK;
+    if (off || (!force && p->shape_asked)) return FIONA_OK;
     if (!hp.n_in || hp.n_in > kGemmMaxInputs || hp.n_out < 2 || ctx->q_max >= (1ull << 50)) return FIONA_OK;
     for (const uint64_t q : ctx->moduli)
         if (q < (1ull << 33)) return FIONA_OK;
