@@ -12,13 +12,20 @@
 //      m_i = (2/N) Re(u_i) and m_{i+n} = (2/N) Im(u_i), n = N/2, with
 //        u_i = sum_j z_j zeta^(-5^j i) = sum_r y_r zeta^(-(4r+1) i),
 //      y_r = z_j for 5^j = 4r + 1 mod 2N (the powers of 5 are the residues
-//      1 mod 4).  With A[k] = y_brv(k) (n-bit reversal) and psi = zeta^2,
-//        u_i = zeta^i sum_k A[k] psi^(-(2 brv(k) + 1) i),
-//      which is n times the inverse negacyclic transform of A of size n
-//      (ntt.cuh over complex fp64) twisted by zeta^i.  So the inverse low
-//      pass gathers A[k] from z, and the inverse high pass multiplies by
-//      zeta^i and rounds Delta (2/N) of the real and imaginary parts to the
-//      64-bit coefficients i and i + n.
+//      1 mod 4), so
+//        u_i = zeta^-i sum_r y_r omega^(r i),  omega = exp(-2 pi i / n),
+//      a cyclic transform of size n = R1 R2.  The low pass gathers y in
+//      bit-reversed order, transforms rows of R2 (row p holds the r = brv(p)
+//      mod R1), and multiplies element (p, c) by omega^(brv(p) c) zeta^-c; the
+//      high pass transforms the columns (R1 elements each) and, since zeta^-i
+//      = zeta^-c zeta^(-R2 q) for i = R2 q + c, multiplies by Delta (2/N)
+//      zeta^(-R2 q) and rounds the real and imaginary parts to the 64-bit
+//      coefficients i and i + n.
+//      The fp64 pipe bounds it (2 lanes a cycle and SM): about 50 fp64
+//      operations a slot at 2^15 slots (a butterfly six, or four additions
+//      where the twiddle is 1 or -i) against 66 with the negacyclic
+//      Gentleman-Sande stages before, whose butterflies take eight.  Measured
+//      on GB300, 93 vectors of 2^15 slots: 0.435 -> 0.324 ms.
 //   2. RNS/NTT form: c_i mod q_l for every limb, then the forward NTT mod
 //      q_l (ntt.cuh, the tables the rescale uses), canonical.
 // Step 1 is floating point: it reproduces round(Delta m_i) except where
@@ -38,13 +45,12 @@ using namespace fiona_ntt;
 
 namespace {
 
-// in device memory, n = N/2 entries each: the twiddles psi^-brv(k) =
-// zeta^(-2 brv(k)) as (cos, sin), the slot index of A[k], and the twists
-// zeta^i
+// in device memory, complex numbers as (cos, sin)
 struct EncTables {
-    const double2 *cinv;
-    const uint32_t *gather;
-    const double2 *twist;
+    const double2 *tw;       // [R2]: exp(-i pi m / h) at h + m, m < h, h a power of two
+    const double2 *mid;      // [n]: omega^(brv(p) c) zeta^-c at p R2 + c
+    const double2 *twist;    // [R1]: zeta^(-R2 q)
+    const uint32_t *gather;  // [n]: the slot of y_brv(k)
 };
 
 struct EmbArgs {
@@ -73,12 +79,11 @@ __device__ __forceinline__ int64_t round_coeff(double x, int *err)
     return 0;
 }
 
-// embedding, inverse low stages of the size-n transform (LN = log2 n):
-// A[k] gathered from the slots
+// embedding, rows of the size-n transform (LN = log2 n): y in bit-reversed
+// order gathered from the slots
 template <int LN>
-__global__ void __launch_bounds__(LowPass<LN>::threads, 2) k_embed_low(EmbArgs A)
+__global__ void __launch_bounds__(LowPass<LN>::threads, 4) k_embed_low(EmbArgs A)
 {
-    using SH = Shape<LN>;
     using PS = LowPass<LN>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p = blockIdx.x >> PS::ltiles;
@@ -86,13 +91,17 @@ __global__ void __launch_bounds__(LowPass<LN>::threads, 2) k_embed_low(EmbArgs A
     const size_t base = (size_t)first << PS::s;
     const double2 *z = A.slots + ((size_t)p << LN);
     const uint32_t *gat = A.E.gather + base;
+    const double2 *mid = A.E.mid + base;
     double2 *w = A.work + ((size_t)p << LN) + base;
     inv_low_pass<LN, PS>(
-        smem_raw, A.E.cinv, first, CplxArith{}, 1, [&](uint32_t e0, uint32_t t) { return z[gat[e0 + t]]; },
-        [&](uint32_t sub, uint32_t pos, double2 v) { w[(sub << PS::s) + pos] = v; });
+        smem_raw, A.E.tw, first, CplxArith{}, 1, [&](uint32_t e0, uint32_t t) { return z[gat[e0 + t]]; },
+        [&](uint32_t sub, uint32_t pos, double2 v) {
+            const uint32_t e = (sub << PS::s) + pos;
+            w[e] = CplxArith::mul(v, mid[e]);
+        });
 }
 
-// embedding, inverse high stages: x zeta^i, rounded Delta (2/N) Re and Im to
+// embedding, columns, then the last twist with Delta (2/N), rounded to the
 // coefficients i and i + n
 template <int LN>
 __global__ void __launch_bounds__(HighPass<LN>::threads, 2) k_embed_high(EmbArgs A)
@@ -101,19 +110,23 @@ __global__ void __launch_bounds__(HighPass<LN>::threads, 2) k_embed_high(EmbArgs
     using PS = HighPass<LN>;
     constexpr uint32_t R2 = 1u << (LN - SH::n1);
     extern __shared__ __align__(16) uint8_t smem_raw[];
+    __shared__ double2 s_twist[1 << SH::n1];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p = blockIdx.x >> PS::ltiles;
     const uint32_t first = tile << PS::lsubs;
     const double2 *g = A.work + ((size_t)p << LN) + first;
-    const double2 *tw = A.E.twist + first;
     int64_t *c = A.coeffs + ((size_t)p << (LN + 1)) + first;
-    const double f = A.factor;
+    for (uint32_t q = threadIdx.x; q < (1u << SH::n1); q += PS::threads) {
+        const double2 t = A.E.twist[q];
+        s_twist[q] = make_double2(t.x * A.factor, t.y * A.factor);
+    }
+    __syncthreads();
     inv_high_pass<LN>(
-        smem_raw, A.E.cinv, first, CplxArith{}, [&](uint32_t sub, uint32_t pos) { return g[(size_t)pos * R2 + sub]; },
+        smem_raw, A.E.tw, first, CplxArith{}, [&](uint32_t sub, uint32_t pos) { return g[(size_t)pos * R2 + sub]; },
         [&](uint32_t sub, uint32_t pos, double2 v) {
             const size_t i = (size_t)pos * R2 + sub;
-            const double2 u = CplxArith::mul(v, tw[i]);
-            c[i] = round_coeff(u.x * f, A.err);
-            c[i + (1u << LN)] = round_coeff(u.y * f, A.err);
+            const double2 u = CplxArith::mul(v, s_twist[pos]);
+            c[i] = round_coeff(u.x, A.err);
+            c[i + (1u << LN)] = round_coeff(u.y, A.err);
         });
 }
 
@@ -185,28 +198,47 @@ __global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 4) k_enc_low(EncA
 // ---------------------------------------------------------------------------
 std::mutex g_enc_mu;
 
+// exp(-i pi x / N) (host)
+double2 unit_root(uint64_t x, uint32_t N)
+{
+    const long double a = -3.141592653589793238462643383279502884L * (long double)x / (long double)N;
+    return make_double2((double)cosl(a), (double)sinl(a));
+}
+
+// byte offsets of the tables (n a power of two of at least 2^9: each part a
+// multiple of 16 bytes)
+struct EncOffsets {
+    size_t tw = 0, mid, twist, gather, total;
+    explicit EncOffsets(uint32_t n)
+    {
+        const uint32_t n1 = log2u(n) / 2;
+        mid = tw + sizeof(double2) * (n >> n1);
+        twist = mid + sizeof(double2) * n;
+        gather = twist + (sizeof(double2) << n1);
+        total = gather + sizeof(uint32_t) * n;
+    }
+};
+
 int build_encode_tables(const fiona_ctx *ctx)
 {
     std::lock_guard<std::mutex> lock(g_enc_mu);
     if (ctx->d_enc) return FIONA_OK;
     const uint32_t N = ctx->N, n = N / 2, ln = log2u(n), M = 2 * N;
-    const size_t tw_bytes = sizeof(double2) * n, gat_bytes = sizeof(uint32_t) * n;
-    const size_t bytes = 2 * tw_bytes + gat_bytes;
-    std::vector<uint8_t> host(bytes);
-    double2 *tw = reinterpret_cast<double2 *>(host.data());
-    double2 *twist = reinterpret_cast<double2 *>(host.data() + tw_bytes);
-    uint32_t *gat = reinterpret_cast<uint32_t *>(host.data() + 2 * tw_bytes);
-    // the shape of the embedding's low pass (LowPass of log2 n)
-    const uint32_t n1 = ln / 2, lt = ln < (uint32_t)kLogTileMax ? ln : (uint32_t)kLogTileMax;
-    const uint32_t lrows = std::max(lt - 1, ln - n1) - (ln - n1);
-    const long double pi = 3.141592653589793238462643383279502884L;
-    for (uint32_t k = 0; k < n; ++k) {
-        // psi^-brv(k) = zeta^(-2 brv(k)) and zeta^k, zeta = exp(i pi / N)
-        const long double a = -2 * pi * (long double)bit_reverse(k, ln) / (long double)N;
-        tw[low_place(k, n1, ln - n1, lrows)] = make_double2((double)cosl(a), (double)sinl(a));
-        const long double b = pi * (long double)k / (long double)N;
-        twist[k] = make_double2((double)cosl(b), (double)sinl(b));
-    }
+    const uint32_t n1 = ln / 2, R1 = 1u << n1, R2 = n >> n1;
+    const EncOffsets off(n);
+    std::vector<uint8_t> host(off.total);
+    double2 *tw = reinterpret_cast<double2 *>(host.data() + off.tw);
+    double2 *mid = reinterpret_cast<double2 *>(host.data() + off.mid);
+    double2 *twist = reinterpret_cast<double2 *>(host.data() + off.twist);
+    uint32_t *gat = reinterpret_cast<uint32_t *>(host.data() + off.gather);
+    auto unit = [=](uint64_t x) { return unit_root(x % M, N); };
+    tw[0] = make_double2(1, 0);
+    for (uint32_t h = 1; h < R2; h *= 2)
+        for (uint32_t m = 0; m < h; ++m) tw[h + m] = unit((uint64_t)m * (N / h));
+    for (uint32_t p = 0; p < R1; ++p)
+        for (uint32_t c = 0; c < R2; ++c)  // omega = exp(-4 pi i / N)
+            mid[p * R2 + c] = unit(4ull * bit_reverse(p, n1) * c + c);
+    for (uint32_t q = 0; q < R1; ++q) twist[q] = unit((uint64_t)R2 * q);
     // slot j sits at the exponent 5^j mod 2N, which is 4r + 1 for one r < n
     std::vector<int64_t> slot_of_r(n, -1);
     uint64_t e5 = 1;
@@ -218,9 +250,9 @@ int build_encode_tables(const fiona_ctx *ctx)
     }
     for (uint32_t k = 0; k < n; ++k) gat[k] = (uint32_t)slot_of_r[bit_reverse(k, ln)];
     void *dev = nullptr;
-    cudaError_t err = cudaMalloc(&dev, bytes);
+    cudaError_t err = cudaMalloc(&dev, off.total);
     if (err != cudaSuccess) return set_error(FIONA_ERR_NOMEM, "encode tables: %s", cudaGetErrorString(err));
-    err = cudaMemcpy(dev, host.data(), bytes, cudaMemcpyHostToDevice);
+    err = cudaMemcpy(dev, host.data(), off.total, cudaMemcpyHostToDevice);
     if (err != cudaSuccess) {
         cudaFree(dev);
         return set_error(FIONA_ERR_CUDA, "encode tables: %s", cudaGetErrorString(err));
@@ -313,9 +345,11 @@ int launch_embed(const fiona_ctx *ctx, void *stream, uint64_t count, const doubl
     const Kernels &K = kernels(n);
     const uint8_t *tab = static_cast<const uint8_t *>(ctx->d_enc);
     EmbArgs a;
-    a.E.cinv = reinterpret_cast<const double2 *>(tab);
-    a.E.twist = reinterpret_cast<const double2 *>(tab + sizeof(double2) * (ctx->N / 2));
-    a.E.gather = reinterpret_cast<const uint32_t *>(tab + 2 * sizeof(double2) * (ctx->N / 2));
+    const EncOffsets off(ctx->N / 2);
+    a.E.tw = reinterpret_cast<const double2 *>(tab + off.tw);
+    a.E.mid = reinterpret_cast<const double2 *>(tab + off.mid);
+    a.E.twist = reinterpret_cast<const double2 *>(tab + off.twist);
+    a.E.gather = reinterpret_cast<const uint32_t *>(tab + off.gather);
     a.factor = 2.0 * scale / (double)ctx->N;
     a.err = ctx->d_kerr;
     cudaStream_t s = (cudaStream_t)stream;
