@@ -184,6 +184,17 @@ uint64_t powm(uint64_t b, uint64_t e, uint64_t q)
     return r;
 }
 
+// x * w mod q for a fixed w, with floor(2^64 w / q): no division a product
+struct FixedMul {
+    uint64_t w, wq, q;
+    FixedMul(uint64_t w_, uint64_t q_) : w(w_), wq((uint64_t)(((u128)w_ << 64) / q_)), q(q_) {}
+    uint64_t operator()(uint64_t x) const
+    {
+        const uint64_t r = x * w - (uint64_t)((u128)x * wq >> 64) * q;  // below 2q
+        return r >= q ? r - q : r;
+    }
+};
+
 // the table entry of w (ntt.cuh): 2^32 w mod q, and both quotients by 2q
 Twiddle twiddle(uint64_t w, uint64_t q)
 {
@@ -211,10 +222,10 @@ uint64_t least_root(uint64_t q, uint32_t N)
         }
     }
     if (!g) return 0;
-    const uint64_t g2 = mulm(g, g, q);
+    const FixedMul by_g2(mulm(g, g, q), q);
     uint64_t best = g, cur = g;
     for (uint32_t j = 1; j < N; ++j) {
-        cur = mulm(cur, g2, q);
+        cur = by_g2(cur);
         best = std::min(best, cur);
     }
     return best;
@@ -251,8 +262,9 @@ int build_tables(const fiona_ctx *ctx)
         // powers of psi, then of psi^-1, placed in bit-reversed order
         for (int dir = 0; dir < 2; ++dir) {
             const uint64_t base = dir == 0 ? psi : powm(psi, q - 2, q);
+            const FixedMul by_base(base, q);
             pw[0] = 1;
-            for (uint32_t i = 1; i < N; ++i) pw[i] = mulm(pw[i - 1], base, q);
+            for (uint32_t i = 1; i < N; ++i) pw[i] = by_base(pw[i - 1]);
             ulonglong2 *d_wv = reinterpret_cast<ulonglong2 *>(host.data() + off + dir * table);
             uint2 *d_om = reinterpret_cast<uint2 *>(host.data() + off + dir * table + wv);
             for (uint32_t k = 0; k < N; ++k) {
