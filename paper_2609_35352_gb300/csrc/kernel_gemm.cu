@@ -6,7 +6,7 @@
 // poly; polys fastest, so that gamma's tile comes from L2 the second time).
 // Per unit, 16 warps
 //   1. read the inputs' residues (each lane one coefficient, coalesced), cut
-//      them into digits and write them to tensor memory;
+//      them into digits and write them to tensor memory, in three parts;
 //   2. per block of 32 outputs, take the 32 signed sums' accumulators, then
 //      those of the two groups of 16 outputs, from tensor memory into
 //      registers (which frees the accumulators for the next multiplications,
@@ -29,9 +29,12 @@
 // issuing warp and the recombination in words, 1.44 with the digit weights
 // read at run time, 1.29 with the signed sums in shared memory, counted unit
 // coordinates and the shorter quotient.  The layer's 3.0 GB take 0.45 ms.
-// Making the next unit's digits under the last group's epilogue (1.44), 112
-// registers a worker by setmaxnreg (1.32) and prefetching gamma's tiles to L1
-// (no change) were not kept.
+// Starting a unit's multiplications when the first third of its digits is
+// there took it from 1.290 to 1.280.  Making the next unit's digits under the
+// last group's epilogue (1.44), 112 registers a worker by setmaxnreg (1.32),
+// prefetching gamma's tiles to L1 (no change), the products by gamma formed
+// with the signed sums (1.31) and additions and shifts in place of some of the
+// recombination's multiplications (1.285 to 1.288) were not kept.
 // All waits are bounded (GemmArgs::wait_ns on the global timer); one that
 // gives up sets the context's error flag and the CTA's abort flag, which ends
 // every other wait, and the CTA frees its tensor memory once its
@@ -110,6 +113,22 @@ __device__ __forceinline__ void issue_signed_n(uint32_t tmem, uint32_t d0, uint3
                      tcs::idesc_f16(128, kGemmBlock), k > 0);
 }
 
+// The same for part `j`, 32 inputs (the last may have 16), of a unit's first
+// block: its digits come in that order.
+template <uint32_t STEPS>
+__device__ __forceinline__ void issue_signed_part(uint32_t tmem, uint32_t d0, uint32_t b, uint32_t j)
+{
+    const uint64_t desc = tcs::smem_desc(b, 128, STEPS * 256) + 32 * j;
+    const uint32_t dig = tmem + 16 * j;
+#pragma unroll
+    for (uint32_t d = 0; d < kDigits; ++d)
+        tcs::mma(tmem + d0 + d * kGemmBlock, dig + 8 * (d * STEPS), desc, tcs::idesc_f16(128, kGemmBlock), j > 0);
+    if (STEPS % 2 && j == STEPS / 2) return;
+#pragma unroll
+    for (uint32_t d = 0; d < kDigits; ++d)
+        tcs::mma(tmem + d0 + d * kGemmBlock, dig + 8 * (d * STEPS + 1), desc + 16, tcs::idesc_f16(128, kGemmBlock), 1);
+}
+
 // (A multiplication's columns all accumulate or are all overwritten: digit 0
 // of the inputs first writes the classes 0 to 5, and the first 16 inputs of
 // digit 5, cut in two, the classes 6 to 10.)
@@ -135,22 +154,26 @@ __device__ __forceinline__ void issue_raw_n(uint32_t tmem, uint32_t d0, uint32_t
     }
 }
 
-#define GEMM_STEPS(F)                                   \
+#define GEMM_STEPS(F, ...)                              \
     switch (steps) {                                    \
-        case 1: F<1>(tmem, d0, b); break;               \
-        case 2: F<2>(tmem, d0, b); break;               \
-        case 3: F<3>(tmem, d0, b); break;               \
-        case 4: F<4>(tmem, d0, b); break;               \
-        case 5: F<5>(tmem, d0, b); break;               \
-        default: F<6>(tmem, d0, b); break;              \
+        case 1: F<1>(__VA_ARGS__); break;               \
+        case 2: F<2>(__VA_ARGS__); break;               \
+        case 3: F<3>(__VA_ARGS__); break;               \
+        case 4: F<4>(__VA_ARGS__); break;               \
+        case 5: F<5>(__VA_ARGS__); break;               \
+        default: F<6>(__VA_ARGS__); break;              \
     }
 __device__ __forceinline__ void issue_signed(uint32_t steps, uint32_t tmem, uint32_t d0, uint32_t b)
 {
-    GEMM_STEPS(issue_signed_n)
+    GEMM_STEPS(issue_signed_n, tmem, d0, b)
+}
+__device__ __forceinline__ void issue_signed(uint32_t steps, uint32_t tmem, uint32_t d0, uint32_t b, uint32_t j)
+{
+    GEMM_STEPS(issue_signed_part, tmem, d0, b, j)
 }
 __device__ __forceinline__ void issue_raw(uint32_t steps, uint32_t tmem, uint32_t d0, uint32_t b)
 {
-    GEMM_STEPS(issue_raw_n)
+    GEMM_STEPS(issue_raw_n, tmem, d0, b)
 }
 #undef GEMM_STEPS
 
@@ -252,7 +275,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
     const GemmLayout lay(a.K, a.chunk);
     const uint32_t tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t base = async::smem_addr(sm);
-    const uint32_t bar_a = base + lay.bars, bar_full = bar_a + 8, bar_empty = bar_a + 16, bar_build = bar_a + 24;
+    const uint32_t bar_full = base + lay.bars, bar_empty = bar_full + 8, bar_build = bar_full + 16;
+    const uint32_t bar_a = bar_full + 24;  // + 8 * part of 32 inputs
     const uint32_t d0 = kDigits * (a.K / 2);  // first accumulator column
     const uint32_t per_limb = a.N / kGemmRows * 2;
     const uint32_t u_begin = (uint32_t)((uint64_t)a.units * blockIdx.x / gridDim.x);
@@ -277,7 +301,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
 
     if (tid == 0) {
         s_abort = 0;
-        async::mbar_init(bar_a, kGemmEpilogueWarps);
+        for (uint32_t j = 0; j < kGemmMaxInputs / 32; ++j) async::mbar_init(bar_a + 8 * j, kGemmEpilogueWarps);
         async::mbar_init(bar_full, 1);
         async::mbar_init(bar_empty, kGemmEpilogueWarps);
         async::mbar_init(bar_build, kGemmEpilogueWarps);
@@ -314,7 +338,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
         bool ok = true;
         for (uint32_t u = u_begin; u < u_end && ok; ++u, ++n_unit, un = step(un)) {
             const uint32_t n_out = chunk_outs(un.c);
-            if (!(ok = wait(bar_a, n_unit & 1))) break;
             for (uint32_t o = 0; o < n_out && ok; o += kGemmBlock) {
                 const uint32_t blk = base + (o / kGemmBlock) * lay.block;
                 const uint32_t n_groups = n_out - o > 16 ? 2 : 1;
@@ -322,7 +345,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                     if (n_full && !(ok = wait(bar_empty, (n_full - 1) & 1))) break;
                     tcs::fence_after();
                     __syncwarp();
-                    if (elect_one()) {
+                    if (o == 0 && g == 0) {
+                        uint32_t j = 0;
+                        for (; j < (steps + 1) / 2; ++j) {
+                            if (!(ok = wait(bar_a + 8 * j, n_unit & 1))) break;
+                            tcs::fence_after();
+                            __syncwarp();
+                            if (elect_one()) issue_signed(steps, tmem, d0, blk + 2 * lay.group, j);
+                            __syncwarp();
+                        }
+                        if (j && elect_one()) tcs::commit(bar_full);
+                        if (!ok) {
+                            n_full += j > 0;
+                            break;
+                        }
+                    } else if (elect_one()) {
                         if (g == 0)
                             issue_signed(steps, tmem, d0, blk + 2 * lay.group);
                         else
@@ -467,10 +504,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                         store_digit<4>(t + 4 * (a.K / 2), w[j]);
                         store_digit<5>(t + 5 * (a.K / 2), w[j]);
                     }
+                    if (j < (a.K + 31) / 32) {
+                        tcs::wait_st();
+                        tcs::fence_before();
+                        arrive(bar_a + 8 * j);
+                    }
                 }
-                tcs::wait_st();
-                tcs::fence_before();
-                arrive(bar_a);
             }
             // the next unit's inputs towards L2, and a new tile's gammas
             if (u + 1 < u_end) {

@@ -62,6 +62,7 @@ def workload(plan, n_raw, N, bits, L, seed, fill="uniform"):
     (17, 32, 0.5, 1024, 34, 2, "uniform"),
     (33, 33, 0.4, 1024, 45, 2, "uniform"),
     (64, 48, 1.0, 1024, 50, 2, "max"),
+    (70, 40, 0.5, 1024, 50, 2, "uniform"),
     (96, 49, 0.9, 1024, 50, 2, "max"),
     (96, 96, 0.5, 4096, 50, 2, "uniform"),
     (81, 200, 0.5, 1024, 48, 1, "uniform"),
