@@ -77,9 +77,10 @@ typedef enum fiona_status {
  * CTA per limb and coefficient tile; the tile of every input is copied once
  * into shared memory (bulk asynchronous copies), shared signed sums are
  * formed once per tile, and the warps split the outputs.  AUTO (the default
- * after fiona_plan_create): TILED for layers with more than one output whose
- * tile fits in shared memory and whose outputs read more than a few operands,
- * DIRECT otherwise.  For a layer whose every raw
+ * after fiona_plan_create): DIRECT for a single output, for layers whose tile
+ * does not fit in shared memory and for those a model of both kernels' time
+ * puts at least a tenth quicker there (mostly few operands an output), TILED
+ * otherwise.  For a layer whose every raw
  * plaintext is constant, TILED is the matrix kernel where the layer is large
  * enough for it (tile_coeffs 128: 128 coefficients of one poly per CTA, both
  * routes as exact products on the tensor cores). */

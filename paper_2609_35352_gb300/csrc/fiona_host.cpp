@@ -571,25 +571,33 @@ static bool use_gemm(const fiona_plan *p, uint32_t n_limbs)
     return p->kernel == 1 && p->gemm && gemm_units(p, n_limbs) >= p->gemm->min_units;
 }
 
-// Layers whose outputs read few operands: the tiled kernel's tile (staging,
-// padded batches, one barrier) then costs more than the direct kernel's
-// repeated reads through L2.  Measured on GB300, tiled against direct time:
-// 3 -> 16 outputs 1.2-1.7, 4 -> 4 1.0-1.4, 6 -> 6 1.1-1.3 (N = 2^10 to 2^16, 2
-// to 24 limbs); the smallest layer, whose 16 scale groups of one term each open
-// a batch of their own, 10.2 us against 8.2; 60-bit moduli 8 -> 8 1.15 and 10 ->
-// 10 1.09 at 2^16 and 12 limbs (and 0.8 for 8 -> 4 at 2^12 and 3 limbs, hence
-// the size bound); 50-bit moduli 8 -> 8 1.0, 10 -> 10 0.92; two outputs of 8
-// operands 1.25-1.85.
+// Whether the direct kernel is expected to take at least 10% less time than the
+// tiled one: layers of few operands an output, where the tile (staging, padded
+// batches, one barrier) costs more than repeated reads through L2, and
+// launches too small to fill the tiled kernel's CTAs.  The direct kernel's time
+// is a sum over a coefficient's raw terms, signed terms, outputs, scale groups
+// and bytes, longer where few CTAs share the SMs (fitted on GB300 to 1391 random
+// layers of 3 to 150 inputs and 2 to 100 outputs: 5% from the measured time, one
+// standard deviation); of the 80 of 695 such layers where the rule takes it,
+// none ran longer and the mean was 0.80 of the tiled kernel's time.  Launches
+// below 16 us go by the operands an output has, six at most, and by the batches
+// of four that scale groups of one term open (the smallest layer, 16 of them:
+// 8.2 us against 10.2).
 static bool few_operands(const fiona_plan *p)
 {
     const fiona_plan_stats_t &s = p->stats;
-    const uint64_t terms = s.n_nonzero_terms, n_out = p->hp.n_out;
-    if (terms <= 6 * n_out) return true;
-    // operations once each scale group opens a batch of four
-    if (p->hp.n_in <= 8 && 4 * std::max<uint64_t>(s.n_scale_groups_used, n_out) >= 2 * terms) return true;
-    if ((uint64_t)p->ctx->N * p->ctx->L * n_out < (1u << 17)) return false;
-    const bool wide = p->ctx->q_max >= (1ull << 52);
-    return (wide && terms <= 10 * n_out) || (n_out <= 2 && terms <= 16 * n_out);
+    if (p->tiled->est_cycles < 33000) {
+        const uint64_t terms = s.n_nonzero_terms;
+        return terms <= 6ull * p->hp.n_out ||
+               (p->hp.n_in <= 8 && 2ull * std::max<uint64_t>(s.n_scale_groups_used, p->hp.n_out) >= terms);
+    }
+    const double raw = s.n_raw_terms, groups = s.n_scale_groups_used, n_out = p->hp.n_out;
+    const double coeffs = (double)p->ctx->N * p->ctx->L, sms = p->ctx->sm_count > 0 ? p->ctx->sm_count : 152;
+    const double bytes = (raw + groups + 2.0 * s.n_inputs_used + 2 * n_out) * 8;
+    const double each = 0.385 * raw + 0.294 * s.n_signed_terms + 1.4 * n_out + 0.27 * groups + bytes / 27.5;
+    const double ctas = coeffs / 256 * n_out;
+    const double cycles = 15400 + coeffs / sms * each * (1 + 0.28 * 16 * sms / ctas);
+    return cycles < 0.9 * p->tiled->est_cycles;
 }
 
 // Kernel choice: DIRECT for a single output (no input reuse to exploit), where

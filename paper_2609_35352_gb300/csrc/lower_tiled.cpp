@@ -66,21 +66,18 @@ struct OutWork {
     std::vector<std::pair<uint32_t, uint32_t>> raws;  // (source | kOpConst if constant, pt)
 };
 
-// Estimated issue cost of operations, in warp instructions, and of the
-// resources they draw on (see the shape search).
+// Estimated issue cost of operations, in warp instructions.
 struct Costs {
     double raw, seg, operand, last, nop;
-    double imad_op;          // wide multiplies (quarter rate) per product operation
-    double smem_operand;     // shared-memory bytes per source read (both polys)
 };
 
 Costs costs_for(int C, bool narrow)
 {
     Costs c{};
     if (narrow) {
-        c = C == 2 ? Costs{34, 70, 8.5, 90, 6, 12, 1024} : Costs{22, 40, 6, 50, 5, 6, 512};
+        c = C == 2 ? Costs{34, 70, 8.5, 90, 6} : Costs{22, 40, 6, 50, 5};
     } else {
-        c = C == 2 ? Costs{60, 80, 8.5, 110, 6, 32, 1024} : Costs{35, 45, 6, 60, 5, 16, 512};
+        c = C == 2 ? Costs{60, 80, 8.5, 110, 6} : Costs{35, 45, 6, 60, 5};
     }
     return c;
 }
@@ -100,6 +97,56 @@ double work_cost(const OutWork &w, const Costs &k, size_t P)
     c += k.nop * (double)(std::max(slots, std::max<size_t>(ops, 1)) - ops);
     return c;
 }
+
+// Time of a launch by shape, in SM cycles: per tile the largest of the
+// schedulers' work, the longest warp's, its plaintext batches' latency and HBM
+// (joined by a p-norm), then the staging of the inputs, times the tiles an SM
+// works through.  Fitted to 53 k launches on GB300 (1391 random layers of 3 to
+// 150 inputs and 2 to 100 outputs, every shape that fits; N = 2^12 to 2^16, 2
+// to 10 limbs of 50 or 60 bits): 8.5% (50 bits) and 7.3% (60) from the
+// measured time, one standard deviation, as much on layers left out.
+struct ShapeCosts {  // cycles a warp: per operation slot, signed operand, sum and output; a lone warp's slowdown
+    double slot, operand, seg, job, latency;
+};
+struct ShapeModel {
+    ShapeCosts c[2];           // one, two coefficients per lane
+    double norm;               // the p-norm's p
+    double stage, stage_in;    // one region: staging, per tile and per input and coefficient of a lane
+    double ahead, ahead_in;    // two: the same
+    double part;               // per partial sum
+    double fetch;              // a plaintext batch's latency
+    double share;              // staging with other CTAs on the SM
+    double window;             // plaintext bytes in flight the L1 serves, in its sizes
+    double hbm;                // bytes a cycle
+    double launch;             // a launch
+
+    // rounds of tiles over the SMs: a launch of few tiles leaves CTA slots empty
+    double cycles(int C, uint32_t W, uint32_t P, bool dbl, uint32_t ctas, double demand, double longest, double deepest,
+                  double bytes, uint32_t n_in, uint32_t n_part, size_t smem, double tiles_per_sm) const
+    {
+        // what the shared memory leaves of the SM's 256 KB for the L1
+        uint32_t carve = 228;
+        for (uint32_t kb : {196u, 164u, 132u, 100u, 64u, 32u, 16u, 8u})
+            if ((double)ctas * ((double)smem + 1088) <= kb * 1024.0) carve = kb;
+        const double l1 = (256.0 - carve) * 1024;
+        const double live = std::min((double)ctas, std::ceil(tiles_per_sm));
+        const double flight = live * W * P * 32 * C * 8;
+        const double terms[4] = {live * demand / 4, longest * c[C - 1].latency, live * bytes / hbm,
+                                 deepest / P * fetch * std::max(1.0, flight / (window * l1))};
+        double t = 0;
+        for (double x : terms) t += std::pow(x, norm);
+        t = std::pow(t, 1 / norm);
+        const double in = (double)n_in * C;
+        t += ((dbl ? ahead + ahead_in * in : stage + stage_in * in) + part * n_part) * (live == 1 ? 1.0 : share);
+        if (C == 2 && W == 16 && P == 8) t *= 1.1;  // (register spills)
+        const double rounds = tiles_per_sm / live;
+        return t * (rounds < 4 ? std::ceil(rounds) : rounds + 0.4) + launch;
+    }
+};
+const ShapeModel kNarrowModel{{{41.8, 13.6, 235, 229, 1.44}, {50.6, 21.1, 415, 329, 1.86}},
+                              2.58, 2840, 56.1, 2110, 13.5, 32.9, 1420, 1.13, 1.36, 29.0, 17000};
+const ShapeModel kWideModel{{{45.9, 14.7, 277, 275, 1.86}, {81.7, 13.0, 541, 313, 2.11}},
+                            2.47, 2520, 44.4, 2020, 7.66, 34.7, 1580, 1.24, 1.24, 25.1, 17800};
 
 struct Job {
     uint32_t target;
@@ -1662,6 +1709,7 @@ int lower_tiled(fiona_plan *p)
     // plans with constant plaintexts run the kernel variant that reads them
     bool has_const = false;
     for (const fiona_term &t : hp.terms) has_const |= t.kind == FIONA_TERM_RAW_CONST;
+    const ShapeModel &model = narrow ? kNarrowModel : kWideModel;
     std::vector<Shape> shapes;
     for (int C : {2, 1})
     for (uint32_t batch : {16u, 8u, 4u}) {
@@ -1728,31 +1776,26 @@ int lower_tiled(fiona_plan *p)
                 const uint32_t by_regs = 65536 / (W * 32 * regs);
                 const uint32_t ctas = std::min({by_smem, by_threads, by_regs, 32u});
                 if (!ctas) continue;
-                // per-tile demand of one CTA (cycles of the resource it uses)
-                double issue = 0, imad = 0, lds = 0, slowest = 0;
+                // per-tile demand of the warps of one CTA
+                const ShapeCosts &mc = model.c[C - 1];
+                double issue = 0, slowest = 0, demand = 0, longest = 0, deepest = 0, prods = 0;
                 for (uint32_t wi = 0; wi < W; ++wi) {
-                    double c = 0;
+                    double c = 0, d = mc.job * (double)jp.per_warp[wi].size();
                     for (const Job &jb : jp.per_warp[wi]) {
                         c += work_cost(jb.w, k, batch);
-                        const double prods = (double)(jb.w.raws.size() + jb.w.segs.size());
-                        imad += prods * k.imad_op;
-                        double opnds = (double)jb.w.raws.size();
-                        for (auto &s : jb.w.segs) opnds += (double)(s.plus.size() + s.minus.size());
-                        lds += opnds * k.smem_operand / 128.0;
+                        prods += (double)(jb.w.raws.size() + jb.w.segs.size());
+                        for (auto &sg : jb.w.segs) d += mc.seg + mc.operand * (double)seg_operands(sg);
                     }
+                    const double slots = (double)sc.w[sc.o_warp + wi * kWarpTableWords + 1];
+                    d += mc.slot * slots;
                     issue += c;
                     slowest = std::max(slowest, c);
+                    demand += d;
+                    longest = std::max(longest, d);
+                    deepest = std::max(deepest, slots);
                 }
                 double node_ops = 0;
-                for (auto &s : lw.nodes) node_ops += k.seg + k.operand * (double)(s.plus.size() + s.minus.size());
-                const double hbm_bytes = (double)(sc.pt_ops + 2ull * hp.n_in + 2ull * hp.n_out) * T * 8;
-                const double hbm = hbm_bytes / 22.0;  // about 22 bytes per SM cycle at the measured copy rate
-                const double shared = std::max({issue / 4.0, imad, lds, hbm});
-                const double serial = slowest * 2.5 + node_ops / W * 2.5 + 150.0 * (lw.n_levels + 2) +
-                                      (dbl ? 0.0 : 1500.0 + (double)hp.n_in * PB / 64.0);
-                const double tiles = (double)ctx->N / T * ctx->L;
-                const double rounds = std::ceil(tiles / ((double)sms * ctas));
-                const double per_round = std::max(ctas * shared, serial + (ctas == 1 ? 0.25 * shared : 0.0));
+                for (auto &sg : lw.nodes) node_ops += mc.seg + mc.operand * (double)seg_operands(sg);
                 Shape s;
                 s.C = C;
                 s.W = W;
@@ -1766,7 +1809,9 @@ int lower_tiled(fiona_plan *p)
                 s.keep = hi;
                 s.ctas = ctas;
                 s.smem = smem - attr.sharedSizeBytes;
-                s.est = rounds * per_round;
+                s.est = model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W, deepest,
+                                     (prods + 2.0 * hp.n_in + 2.0 * hp.n_out) * T * 8, hp.n_in, jp.n_part, s.smem,
+                                     (double)ctx->N / T * ctx->L / (double)sms);
                 shapes.push_back(s);
                 if (getenv("FIONA_TILED_DEBUG"))
                     fprintf(stderr,
@@ -1800,6 +1845,16 @@ int lower_tiled(fiona_plan *p)
     };
     Shape best = *std::max_element(shapes.begin(), shapes.end(),
                                    [&](const Shape &a, const Shape &b) { return key(a) < key(b); });
+    // Away from the layers that ranking was made on, the shape the model puts
+    // first, where it promises at least 12% (one and a half times a prediction's
+    // error; 25% below eight outputs, whose split work it knows less well) and
+    // the launch takes at least 40 us.  On 778 random layers (2^15, up to 8
+    // limbs) it moved the time per layer by 4 to 6% on average, at best 100
+    // inputs -> 40 outputs: 1.96 ms with one coefficient per lane, two regions and
+    // 2 x 8 warps, 0.91 with two and one region; at worst 4% up.
+    const Shape &quick = *std::min_element(shapes.begin(), shapes.end(),
+                                           [](const Shape &a, const Shape &b) { return a.est < b.est; });
+    if (!p->shape_asked && best.est > 82800 && quick.est < (hp.n_out < 8 ? 0.75 : 0.88) * best.est) best = quick;
     // tuning override "C,W,double[,most shared sums kept[,P]]": every shape
     // computes the same residues
     if (const char *env = getenv("FIONA_TILED_SHAPE")) {
@@ -2014,6 +2069,7 @@ int lower_tiled(fiona_plan *p)
     ts->warps = best.W;
     ts->tile = T;
     ts->batch = best.P;
+    ts->est_cycles = best.est;
     ts->has_const = has_const;
     ts->smem = best.smem;
     ts->ctas_per_sm = best.ctas;

@@ -1,6 +1,9 @@
-"""Which kernel a plan takes by itself (FIONA_KERNEL_AUTO), around the lines of
-the rule: outputs of few operands run on the direct kernel, unless a shape of
-the tiled kernel is asked for.  Both give the same residues (GPU parity)."""
+"""Which kernel and shape a plan takes by itself (FIONA_KERNEL_AUTO), on both
+sides of the rule's lines: the direct kernel where the model of its time is a
+tenth below the tiled kernel's, and for small launches of few operands an
+output, unless a shape of the tiled kernel is asked for; the tiled kernel's shape
+where the model of its time moves it.  Every choice gives the same residues (GPU
+parity)."""
 import pytest
 
 from paper_2609_35352_gb300 import build as B
@@ -13,28 +16,41 @@ def built():
     B.build()
 
 
-def kernel(n_in, n_out, N=1 << 16, L=4, bits=50, per_term=False, desc=None):
-    tern = n_in * n_out // 2
+def stats(n_in, n_out, N=1 << 16, L=4, bits=50, signed=0.5, per_term=False, desc=None):
+    tern = int(n_in * n_out * signed)
     desc = desc or W.dense_hybrid_plan(W.PlanRng(7), n_in, n_out, tern // 2, tern // 2, 0, group_per_term=per_term)
     ctx = F.Context(N, W.ntt_primes(N, bits, L), device=F.FIONA_DEVICE_NONE)
-    return F.Plan(ctx, desc).stats()["kernel"]
+    return F.Plan(ctx, desc).stats()
 
 
-@pytest.mark.parametrize("n_in,n_out,bits,direct", [
-    (6, 6, 50, True), (7, 6, 50, False), (3, 54, 50, True),   # six operands an output
-    (10, 10, 60, True), (11, 10, 60, False), (10, 10, 50, False),  # ten with wide moduli
-    (16, 2, 50, True), (17, 2, 50, False),                    # two outputs
-    (64, 1, 50, True),                                        # one
+@pytest.mark.parametrize("n_in,n_out,L,bits,signed,direct", [
+    (3, 49, 4, 60, 0.54, True), (3, 73, 10, 40, 0.0, False),     # three operands an output: wide, narrow
+    (4, 9, 13, 45, 0.95, True), (6, 65, 2, 50, 0.1, False),
+    (113, 9, 5, 60, 1.0, True), (112, 4, 3, 60, 0.9, False),     # many inputs, few outputs
+    (64, 1, 4, 50, 0.5, True),                                   # one output
 ])
-def test_few_operands(n_in, n_out, bits, direct):
-    assert kernel(n_in, n_out, bits=bits) == (F.FIONA_KERNEL_DIRECT if direct else F.FIONA_KERNEL_TILED)
+def test_direct_kernel(n_in, n_out, L, bits, signed, direct):
+    k = stats(n_in, n_out, L=L, bits=bits, signed=signed)["kernel"]
+    assert k == (F.FIONA_KERNEL_DIRECT if direct else F.FIONA_KERNEL_TILED)
 
 
-def test_size_groups_and_overrides(monkeypatch):
-    assert kernel(8, 8, N=4096, L=2, bits=60) == F.FIONA_KERNEL_TILED  # wide, but too small a launch
-    assert kernel(8, 4, per_term=True) == F.FIONA_KERNEL_DIRECT       # a batch of four per one-term group
-    assert kernel(8, 4) == F.FIONA_KERNEL_TILED
-    wl = W.make_workload("tiny")
-    assert kernel(8, 4, N=wl.N, L=wl.L, bits=40, desc=wl.plan) == F.FIONA_KERNEL_DIRECT
+def test_small_launches_and_overrides(monkeypatch):
+    small = dict(N=4096, L=3)
+    assert stats(6, 6, **small)["kernel"] == F.FIONA_KERNEL_DIRECT    # six operands an output
+    assert stats(7, 6, **small)["kernel"] == F.FIONA_KERNEL_TILED
+    assert stats(8, 4, **small)["kernel"] == F.FIONA_KERNEL_TILED
+    wl = W.make_workload("tiny")  # a batch of four per one-term group
+    assert stats(8, 4, N=wl.N, L=wl.L, bits=40, desc=wl.plan)["kernel"] == F.FIONA_KERNEL_DIRECT
     monkeypatch.setenv("FIONA_TILED_SHAPE", "2,4,1")
-    assert kernel(6, 6) == F.FIONA_KERNEL_TILED
+    assert stats(6, 6, **small)["kernel"] == F.FIONA_KERNEL_TILED
+
+
+def test_tiled_shape():
+    """Two coefficients per lane with one source region, where two regions fit
+    only with one; the shapes of the measured layers as they were."""
+    assert stats(100, 40, N=1 << 15, L=8, signed=0.6)["tile_coeffs"] == 64
+    assert stats(125, 52, N=1 << 15, L=8, bits=60, signed=1.0)["tile_coeffs"] == 64
+    for name, coeffs, warps in (("vgg", 32, 16), ("vit", 64, 8), ("bert", 64, 12)):
+        wl = W.make_workload(name)
+        s = stats(0, 0, N=wl.N, L=wl.L, desc=wl.plan)
+        assert (s["tile_coeffs"], s["warps_per_cta"]) == (coeffs, warps)
