@@ -343,7 +343,8 @@ def measured_peak():
 
 KERNEL_FILES = {"direct": ["kernel_direct.cu", "rns.cuh"],
                 "tiled": ["kernel_tiled.cu", "kernel_tiled_off.cu", "kernel_tiled_w12.cu", "tiled_kernel.cuh", "tiled.h", "lower_tiled.cpp",
-                          "rns.cuh", "tile_math.cuh", "async.cuh", "tc_signed.cuh", "tc_geometry.h", "../build.py"]}
+                          "rns.cuh", "tile_math.cuh", "async.cuh", "tc_signed.cuh", "tc_geometry.h", "../build.py"],
+                "matrix": ["kernel_gemm.cu", "gemm.h", "lower_gemm.cpp", "rns.cuh", "async.cuh", "tc_signed.cuh", "../build.py"]}
 
 
 def kernel_source_hash(kernel: str) -> str:
@@ -534,7 +535,8 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> None:
     avg_kernel_s = statistics.mean(kernel_ms) / 1e3
     peak, peak_kind = measured_peak()
     achieved = stats["bytes_min"] / avg_kernel_s / 1e9
-    kernel = "tiled" if stats["kernel"] == 2 else "direct"
+    # (a tile of 128 coefficients of one poly is the matrix kernel's alone)
+    kernel = "direct" if stats["kernel"] != 2 else "matrix" if stats.get("tile_coeffs") == 128 else "tiled"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak,
                 "peak_nominal": NOMINAL_HBM_GBS, "frac_nominal": achieved / NOMINAL_HBM_GBS,
@@ -620,12 +622,11 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> None:
 # --op rescale
 # ----------------------------------------------------------------------------
 # Integer multiplies (IMAD on the FMA-heavy pipe, 64 per clock per SM) that
-# one forward butterfly needs at least: the quotient estimate (a wide
-# product and two high halves) and the two 64-bit low products (a wide
-# product and two plain multiplies each); a wide product takes two issue
-# slots.  The derived peak: 152 SMs x 64 multiplies per clock x 2070 MHz /
-# 12 slots = 1678 G butterflies/s.
-IMAD_SLOTS_PER_BUTTERFLY = 12
+# one forward butterfly takes: five 32x32 -> 64-bit products (two for the
+# quotient, two for the product by the two-word twiddle, one by the modulus),
+# two issue slots each, and three 32-bit ones.  The derived peak: 152 SMs x 64
+# multiplies per clock x 2070 MHz / 13 slots = 1549 G butterflies/s.
+IMAD_SLOTS_PER_BUTTERFLY = 13
 IMAD_PER_CLK_PER_SM = 64
 SM_COUNT = 152
 SM_MAX_MHZ = 2070.0

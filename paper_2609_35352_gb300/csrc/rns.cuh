@@ -1,7 +1,8 @@
 // rns.cuh -- RNS modular-arithmetic core for residues of primes q < 2^60.
 //
 // Residues are canonical uint64 values in [0, q).  Products of two residues
-// are < 2^120 and are accumulated lazily in 128 bits (lo, hi); the host
+// are < 2^120 and are accumulated lazily in 128 bits (lo, hi), the two middle
+// 32-bit cross products apart where that pays (mac, settle); the host
 // bounds how many products may be added before a reduction (at least 256 for
 // q < 2^60).  Reductions use Barrett's method with constants computed on the
 // host per limb:
