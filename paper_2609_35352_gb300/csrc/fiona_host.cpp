@@ -580,15 +580,16 @@ static bool use_gemm(const fiona_plan *p, uint32_t n_limbs)
 // layers of 3 to 150 inputs and 2 to 100 outputs: 5% from the measured time, one
 // standard deviation); of the 80 of 695 such layers where the rule takes it,
 // none ran longer and the mean was 0.80 of the tiled kernel's time.  Launches
-// below 16 us go by the operands an output has, six at most, and by the batches
-// of four that scale groups of one term open (the smallest layer, 16 of them:
-// 8.2 us against 10.2).
+// below 16 us go by the operands an output has, six at most (3 -> 7 at 2^13 and
+// 5 limbs 10.9 us against 17.1; not two outputs, 4 -> 2 10.9 against 8.8), and by
+// the batches of four that scale groups of one term open (the smallest layer, 16
+// of them: 8.2 us against 10.2).
 static bool few_operands(const fiona_plan *p)
 {
     const fiona_plan_stats_t &s = p->stats;
     if (p->tiled->est_cycles < 33000) {
         const uint64_t terms = s.n_nonzero_terms;
-        return terms <= 6ull * p->hp.n_out ||
+        return (p->hp.n_out > 2 && terms <= 6ull * p->hp.n_out) ||
                (p->hp.n_in <= 8 && 2ull * std::max<uint64_t>(s.n_scale_groups_used, p->hp.n_out) >= terms);
     }
     const double raw = s.n_raw_terms, groups = s.n_scale_groups_used, n_out = p->hp.n_out;

@@ -1704,7 +1704,7 @@ int lower_tiled(fiona_plan *p)
         double balance = 0;           // mean warp cost / largest warp cost
         uint32_t keep = 0, ctas = 0;  // shared sums requested (top of the ranking)
         size_t smem = 0;
-        double est = 0;
+        std::vector<double> level;    // predicted cycles at all limbs, one less, ... half of them
     };
     // plans with constant plaintexts run the kernel variant that reads them
     bool has_const = false;
@@ -1809,15 +1809,17 @@ int lower_tiled(fiona_plan *p)
                 s.keep = hi;
                 s.ctas = ctas;
                 s.smem = smem - attr.sharedSizeBytes;
-                s.est = model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W, deepest,
+                for (uint32_t n = ctx->L; 2 * n >= ctx->L && n; --n)
+                    s.level.push_back(
+                        model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W, deepest,
                                      (prods + 2.0 * hp.n_in + 2.0 * hp.n_out) * T * 8, hp.n_in, jp.n_part, s.smem,
-                                     (double)ctx->N / T * ctx->L / (double)sms);
+                                     (double)ctx->N / T * n / (double)sms));
                 shapes.push_back(s);
                 if (getenv("FIONA_TILED_DEBUG"))
                     fprintf(stderr,
                             "C=%d P=%u W=%u dbl=%d w12=%d keep=%u sched=%zu parts=%u smem=%zu ctas=%u pad=%.2f est=%.0f\n",
                             C, batch, W, (int)dbl, (int)w12, s.keep, sc.w.size() * 4, jp.n_part, smem, ctas, s.pad,
-                            s.est);
+                            s.level[0]);
             }
         }
     }
@@ -1841,7 +1843,7 @@ int lower_tiled(fiona_plan *p)
         const bool deep = s.w12 && s.W == 12 && s.P == 8 && s.balance >= 0.95;
         const int pref = s.C == 2 ? (deep ? 3 : s.P == 4 ? 2 : 1) : (s.P == 16 ? 2 : s.P == 8 ? 1 : 0);
         const uint32_t resident = deep ? 16 : std::min<uint32_t>(s.ctas * s.W, 16);
-        return std::make_tuple(s.dbl ? 1 : 0, resident, s.C, s.ctas, pref, -s.est);
+        return std::make_tuple(s.dbl ? 1 : 0, resident, s.C, s.ctas, pref, -s.level[0]);
     };
     Shape best = *std::max_element(shapes.begin(), shapes.end(),
                                    [&](const Shape &a, const Shape &b) { return key(a) < key(b); });
@@ -1852,9 +1854,17 @@ int lower_tiled(fiona_plan *p)
     // limbs) it moved the time per layer by 4 to 6% on average, at best 100
     // inputs -> 40 outputs: 1.96 ms with one coefficient per lane, two regions and
     // 2 x 8 warps, 0.91 with two and one region; at worst 4% up.
-    const Shape &quick = *std::min_element(shapes.begin(), shapes.end(),
-                                           [](const Shape &a, const Shape &b) { return a.est < b.est; });
-    if (!p->shape_asked && best.est > 82800 && quick.est < (hp.n_out < 8 ? 0.75 : 0.88) * best.est) best = quick;
+    // It has to be no slower at lower levels too, down to half the limbs, where a
+    // launch of few rounds of tiles may end in a nearly empty one (24 -> 26 at
+    // 2^12: three CTAs of 4 warps an SM, quicker at 14 limbs, took 40.8 us
+    // against 30.8 at 9).
+    const Shape *quick = nullptr;
+    for (const Shape &a : shapes) {
+        bool ok = a.level[0] < (hp.n_out < 8 ? 0.75 : 0.88) * best.level[0];
+        for (size_t i = 1; i < a.level.size(); ++i) ok &= a.level[i] <= 1.03 * best.level[i];
+        if (ok && (!quick || a.level[0] < quick->level[0])) quick = &a;
+    }
+    if (!p->shape_asked && best.level[0] > 82800 && quick) best = Shape(*quick);
     // tuning override "C,W,double[,most shared sums kept[,P]]": every shape
     // computes the same residues
     if (const char *env = getenv("FIONA_TILED_SHAPE")) {
@@ -2069,7 +2079,7 @@ int lower_tiled(fiona_plan *p)
     ts->warps = best.W;
     ts->tile = T;
     ts->batch = best.P;
-    ts->est_cycles = best.est;
+    ts->est_cycles = best.level[0];
     ts->has_const = has_const;
     ts->smem = best.smem;
     ts->ctas_per_sm = best.ctas;

@@ -38,6 +38,7 @@ def test_small_launches_and_overrides(monkeypatch):
     small = dict(N=4096, L=3)
     assert stats(6, 6, **small)["kernel"] == F.FIONA_KERNEL_DIRECT    # six operands an output
     assert stats(7, 6, **small)["kernel"] == F.FIONA_KERNEL_TILED
+    assert stats(4, 2, **small)["kernel"] == F.FIONA_KERNEL_TILED     # two outputs
     assert stats(8, 4, **small)["kernel"] == F.FIONA_KERNEL_TILED
     wl = W.make_workload("tiny")  # a batch of four per one-term group
     assert stats(8, 4, N=wl.N, L=wl.L, bits=40, desc=wl.plan)["kernel"] == F.FIONA_KERNEL_DIRECT
