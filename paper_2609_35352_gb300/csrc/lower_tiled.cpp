@@ -1848,8 +1848,10 @@ int lower_tiled(fiona_plan *p)
     Shape best = *std::max_element(shapes.begin(), shapes.end(),
                                    [&](const Shape &a, const Shape &b) { return key(a) < key(b); });
     // Away from the layers that ranking was made on, the shape the model puts
-    // first, where it promises at least 12% (one and a half times a prediction's
-    // error; 25% below eight outputs, whose split work it knows less well) and
+    // first, where it promises more than 1.65 times a prediction's error (14%, and
+    // 12% with wide moduli; with 12% for both one layer in 600, 11 -> 63 of 50
+    // bits at 2^13, became 5% slower; 25% below eight outputs, whose split work
+    // it knows less well) and
     // the launch takes at least 40 us.  On 778 random layers (2^15, up to 8
     // limbs) it moved the time per layer by 4 to 6% on average, at best 100
     // inputs -> 40 outputs: 1.96 ms with one coefficient per lane, two regions and
@@ -1858,9 +1860,10 @@ int lower_tiled(fiona_plan *p)
     // launch of few rounds of tiles may end in a nearly empty one (24 -> 26 at
     // 2^12: three CTAs of 4 warps an SM, quicker at 14 limbs, took 40.8 us
     // against 30.8 at 9).
+    const double margin = hp.n_out < 8 ? 0.75 : narrow ? 0.86 : 0.88;
     const Shape *quick = nullptr;
     for (const Shape &a : shapes) {
-        bool ok = a.level[0] < (hp.n_out < 8 ? 0.75 : 0.88) * best.level[0];
+        bool ok = a.level[0] < margin * best.level[0];
         for (size_t i = 1; i < a.level.size(); ++i) ok &= a.level[i] <= 1.03 * best.level[i];
         if (ok && (!quick || a.level[0] < quick->level[0])) quick = &a;
     }
