@@ -43,6 +43,7 @@ constexpr uint32_t kGemmMaxRaw = 64;        // raw terms per output
 constexpr uint32_t kGemmEpilogueWarps = 16; // and one warp that issues the multiplications
 constexpr uint32_t kGemmThreads = (kGemmEpilogueWarps + 1) * 32;
 constexpr uint32_t kGemmNoGamma = 0xffffffffu;
+constexpr uint32_t kGemmTestDigits = 1, kGemmTestFull = 2;  // the digits' barriers; the accumulators'
 
 // one entry of G or W: output (in its chunk) and input; a raw entry's plaintext
 struct GemmTerm {
@@ -64,7 +65,8 @@ struct GemmArgs {
     uint32_t chunk;              // outputs per chunk (a multiple of 32)
     uint32_t n_chunks;
     uint32_t units;              // chunks x limbs x coefficient tiles x polys
-    uint64_t wait_ns;
+    uint64_t wait_ns;            // bound of every wait
+    uint32_t test_flags;         // test only: barriers that expect an arrival too many (kGemmTest...)
     // 1, 2^8, 2^16, 2^24, read at run time: multiplications by literal powers
     // of two become several shifts and additions
     uint32_t c1, c8, c16, c24;

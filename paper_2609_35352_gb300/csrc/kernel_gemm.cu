@@ -30,14 +30,16 @@
 // read at run time, 1.29 with the signed sums in shared memory, counted unit
 // coordinates and the shorter quotient.  The layer's 3.0 GB take 0.45 ms.
 // Starting a unit's multiplications when the first third of its digits is
-// there took it from 1.290 to 1.280.  Making the next unit's digits under the
+// there took it from 1.290 to 1.280; leaving the waits as whole warps, to 1.288
+// (below).  Making the next unit's digits under the
 // last group's epilogue (1.44), 112 registers a worker by setmaxnreg (1.32),
 // prefetching gamma's tiles to L1 (no change), the products by gamma formed
 // with the signed sums (1.31) and additions and shifts in place of some of the
 // recombination's multiplications (1.285 to 1.288) were not kept.
 // All waits are bounded (GemmArgs::wait_ns on the global timer); one that
 // gives up sets the context's error flag and the CTA's abort flag, which ends
-// every other wait, and the CTA frees its tensor memory once its
+// every other wait; each warp then stops as a whole, at the end of its unit or
+// of a build barrier, and the CTA frees its tensor memory once its
 // multiplications in flight have completed.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -267,6 +269,18 @@ constexpr uint64_t kSplitB1 = 1ull << 50;
 // x mod q, x < 2^64
 __device__ __forceinline__ uint64_t mod64(uint64_t x, const LimbConst &m) { return rns::reduce64(x, m); }
 
+// A wait whose first try found the phase incomplete.  Giving up (or finding
+// that another thread did) leaves `*abort` set; the caller goes on either way and
+// looks at the flag where its whole warp can leave.  Out of line: inline, the
+// clock and the loops took the 96 -> 96 layer from 1.278 to 1.347 ms.
+__device__ __noinline__ void slow_wait(uint32_t bar, uint32_t parity, int *abort, uint64_t limit_ns, int *err)
+{
+    volatile int *flag = abort;
+    if (*flag || async::mbar_wait_bounded(bar, parity, flag, limit_ns) || *flag) return;
+    *flag = 1;
+    atomicOr(err, 1);
+}
+
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
 {
     extern __shared__ __align__(128) char sm[];
@@ -276,6 +290,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
     const uint32_t tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t base = async::smem_addr(sm);
     const uint32_t bar_full = base + lay.bars, bar_empty = bar_full + 8, bar_build = bar_full + 16;
+    const uint32_t bar_drain = bar_full + 48;
     const uint32_t bar_a = bar_full + 24;  // + 8 * part of 32 inputs
     const uint32_t d0 = kDigits * (a.K / 2);  // first accumulator column
     const uint32_t per_limb = a.N / kGemmRows * 2;
@@ -301,8 +316,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
 
     if (tid == 0) {
         s_abort = 0;
-        for (uint32_t j = 0; j < kGemmMaxInputs / 32; ++j) async::mbar_init(bar_a + 8 * j, kGemmEpilogueWarps);
-        async::mbar_init(bar_full, 1);
+        for (uint32_t j = 0; j < kGemmMaxInputs / 32; ++j)
+            async::mbar_init(bar_a + 8 * j, kGemmEpilogueWarps + ((a.test_flags & kGemmTestDigits) != 0));
+        async::mbar_init(bar_full, 1 + ((a.test_flags & kGemmTestFull) != 0));
+        async::mbar_init(bar_drain, 1);
         async::mbar_init(bar_empty, kGemmEpilogueWarps);
         async::mbar_init(bar_build, kGemmEpilogueWarps);
         async::mbar_init_fence();
@@ -313,14 +330,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
     tcs::fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
 
-    auto wait = [&](uint32_t bar, uint32_t parity) {
-        if (async::mbar_wait_bounded(bar, parity, &s_abort, a.wait_ns)) return true;
-        if (!s_abort) {
-            s_abort = 1;
-            atomicOr(a.err, 1);
-        }
-        return false;
+    // Waits.  Each lane has its own clock and its own look at the abort flag, and
+    // one that left alone would leave the others at a warp-wide instruction: so
+    // no wait leaves a loop.  After one that gave up a warp goes on with whatever
+    // the operands hold (no address depends on them) and leaves by a vote, at the
+    // end of the unit or of a build barrier, which s_gamma's entries depend on.
+    auto pass = [&](uint32_t bar, uint32_t parity) {  // (a __syncwarp follows)
+        if (!async::mbar_try_wait(bar, parity)) slow_wait(bar, parity, &s_abort, a.wait_ns, a.err);
     };
+    auto pass_warp = [&](uint32_t bar, uint32_t parity) {
+        if (!__all_sync(0xffffffffu, async::mbar_try_wait(bar, parity)))
+            slow_wait(bar, parity, &s_abort, a.wait_ns, a.err);
+        __syncwarp();
+    };
+    auto going = [&] { return __all_sync(0xffffffffu, *(volatile int *)&s_abort == 0) != 0; };
     // one arrival per warp
     auto arrive = [&](uint32_t bar) {
         __syncwarp();
@@ -338,27 +361,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
         bool ok = true;
         for (uint32_t u = u_begin; u < u_end && ok; ++u, ++n_unit, un = step(un)) {
             const uint32_t n_out = chunk_outs(un.c);
-            for (uint32_t o = 0; o < n_out && ok; o += kGemmBlock) {
+            for (uint32_t o = 0; o < n_out; o += kGemmBlock) {
                 const uint32_t blk = base + (o / kGemmBlock) * lay.block;
                 const uint32_t n_groups = n_out - o > 16 ? 2 : 1;
                 for (uint32_t g = 0; g <= n_groups; ++g, ++n_full) {
-                    if (n_full && !(ok = wait(bar_empty, (n_full - 1) & 1))) break;
+                    if (n_full) pass(bar_empty, (n_full - 1) & 1);
                     tcs::fence_after();
                     __syncwarp();
                     if (o == 0 && g == 0) {
-                        uint32_t j = 0;
-                        for (; j < (steps + 1) / 2; ++j) {
-                            if (!(ok = wait(bar_a + 8 * j, n_unit & 1))) break;
+                        for (uint32_t j = 0; j < (steps + 1) / 2; ++j) {
+                            pass(bar_a + 8 * j, n_unit & 1);
                             tcs::fence_after();
                             __syncwarp();
                             if (elect_one()) issue_signed(steps, tmem, d0, blk + 2 * lay.group, j);
                             __syncwarp();
                         }
-                        if (j && elect_one()) tcs::commit(bar_full);
-                        if (!ok) {
-                            n_full += j > 0;
-                            break;
-                        }
+                        if (elect_one()) tcs::commit(bar_full);
                     } else if (elect_one()) {
                         if (g == 0)
                             issue_signed(steps, tmem, d0, blk + 2 * lay.group);
@@ -369,12 +387,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                     __syncwarp();
                 }
             }
+            ok = going();
         }
-        // the multiplications in flight complete before the tensor memory goes
-        if (!ok && n_full) {
-            const int never = 0;
-            async::mbar_wait_bounded(bar_full, (n_full - 1) & 1, &never, kDrainNs);
-        }
+        // every multiplication issued completes before the tensor memory goes,
+        // whoever gave up
+        const int never = 0;
+        if (elect_one()) tcs::commit(bar_drain);
+        __syncwarp();
+        async::mbar_wait_bounded(bar_drain, 0, &never, kDrainNs);
+        __syncwarp();
     } else {
         // ---- digits, epilogue
         const uint32_t q4 = warp & 3, k4 = warp >> 2;  // tensor memory quarter; share of the inputs and outputs
@@ -395,7 +416,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
         const uint32_t stride = a.L * a.N * 8;  // bytes between polys (at most 2^26)
         auto build_barrier = [&] {
             arrive(bar_build);
-            return wait(bar_build, n_build++ & 1);
+            pass_warp(bar_build, n_build++ & 1);
+            return going();
         };
         for (uint32_t u = u_begin; u < u_end && ok; ++u) {
             const Unit v = un;
@@ -530,9 +552,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
             // 2. the blocks of outputs
             const char *gam = reinterpret_cast<const char *>(a.pt + (size_t)l * a.N + k0 + 32 * q4 + lane);
             char *y = reinterpret_cast<char *>(a.out + ((size_t)(out0 * 2 + poly) * a.L + l) * a.N + k0 + 32 * q4 + lane);
-            for (uint32_t o = 0; o < n_out && ok; o += kGemmBlock) {
+            for (uint32_t o = 0; o < n_out; o += kGemmBlock) {
                 const uint32_t n_groups = n_out - o > 16 ? 2 : 1;
-                if (!(ok = wait(bar_full, n_full++ & 1))) break;
+                pass_warp(bar_full, n_full++ & 1);
                 tcs::fence_after();
                 {
                     uint32_t e[2][kDigits][4];
@@ -571,7 +593,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                         gm[i] = gi[i] != kGemmNoGamma
                                     ? __ldg(reinterpret_cast<const uint64_t *>(gam + (uint64_t)gi[i] * stride))
                                     : 0;
-                    if (!(ok = wait(bar_full, n_full++ & 1))) break;
+                    pass_warp(bar_full, n_full++ & 1);
                     tcs::fence_after();
                     char *yo = y + (uint64_t)(o1 * 2) * stride;
                     uint32_t e[kClasses][4];
@@ -603,6 +625,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                     }
                 }
             }
+            ok = going();
         }
     }
     tcs::fence_before();

@@ -97,6 +97,10 @@ int lower_gemm(fiona_plan *p)
     a.chunk = chunk;
     a.n_chunks = n_chunks;
     a.wait_ns = 2000000000ull;
+    if (const char *t = getenv("FIONA_TEST_GEMM_TIMEOUT")) {  // test only: a wait that runs out
+        a.test_flags = (uint32_t)atoi(t) & (kGemmTestDigits | kGemmTestFull);
+        if (a.test_flags) a.wait_ns = 2000000ull;
+    }
     a.c1 = 1;
     a.c8 = 1u << 8;
     a.c16 = 1u << 16;

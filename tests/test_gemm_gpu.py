@@ -143,3 +143,30 @@ def test_matrix_kernel_levels_and_choice(monkeypatch):
     assert tile(W.build_plan(3, 2, rows, 3, [1, 2], [0, 0], [], [])) < 128
     monkeypatch.setenv("FIONA_CONST_GEMM", "0")
     assert tile(plan) < 128
+
+
+@pytest.mark.parametrize("late", [1, 2])
+def test_matrix_kernel_wait_runs_out(late, monkeypatch):
+    """A test-only plan (FIONA_TEST_GEMM_TIMEOUT) with waits bounded at 2 ms and
+    barriers that expect one arrival too many: those of the digits (1: the
+    issuing warp's wait runs out) or that of the accumulators (2: the workers'
+    wait does, and the issuing warp has multiplications to wait for).  The CTA
+    stops and frees its tensor memory, fiona_device_check reports FIONA_ERR_TIMEOUT
+    once, and the next evaluation on the same context is exact."""
+    monkeypatch.setenv("FIONA_CONST_GEMM", "1")
+    monkeypatch.setenv("FIONA_TEST_GEMM_TIMEOUT", str(late))
+    plan, n_raw = layer(40, 33, 0.5, 11)
+    wl = workload(plan, n_raw, 1024, 50, 2, 17)
+    dl = DeviceLayer(wl)
+    dl.plan.select_kernel("tiled")
+    assert dl.plan.stats()["tile_coeffs"] == 128
+    dl.run()
+    torch.cuda.synchronize()
+    assert dl.ctx.device_check() == F.FIONA_ERR_TIMEOUT
+    assert dl.ctx.device_check() == F.FIONA_OK  # the flag was cleared
+    monkeypatch.delenv("FIONA_TEST_GEMM_TIMEOUT")
+    p = F.Plan(dl.ctx, plan)
+    p.select_kernel("tiled")
+    p.eval(dl.d_in, dl.d_pt, dl.d_out)
+    assert np.array_equal(dl.outputs(), oracle.linear_eval(plan, wl.moduli, dl.X, dl.P))
+    assert dl.ctx.device_check() == F.FIONA_OK
