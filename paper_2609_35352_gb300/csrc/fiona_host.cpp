@@ -36,6 +36,24 @@ static int cuda_fail(cudaError_t e, const char *what)
     return set_error(FIONA_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// The limit is one setting per kernel and device, and every plan that runs the
+// kernel launches under it: so it goes to the device's most (less the kernel's
+// static part), the same whichever plan asks.  It only admits launches; what
+// one occupies goes by its own size.
+int allow_shared_memory(const void *kernel, size_t bytes, const char *what)
+{
+    int device = 0, optin = 0;
+    cudaFuncAttributes attr;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, kernel);
+    if (e != cudaSuccess) return cuda_fail(e, what);
+    if (attr.sharedSizeBytes + bytes > (size_t)optin)
+        return set_error(FIONA_ERR_CUDA, "%s: %zu bytes of shared memory", what, attr.sharedSizeBytes + bytes);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)attr.sharedSizeBytes);
+    return e == cudaSuccess ? FIONA_OK : cuda_fail(e, what);
+}
+
 extern "C" const char *fiona_last_error(void) { return g_last_error; }
 
 extern "C" int fiona_abi_version(void) { return FIONA_ABI_VERSION; }

@@ -150,4 +150,7 @@ int launch_encode_coeffs(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64
 void free_encode_tables(const fiona_ctx *ctx);
 
 // fiona_host.cpp
+// lets launches of `kernel` on the current device have `bytes` of dynamic
+// shared memory
+int allow_shared_memory(const void *kernel, size_t bytes, const char *what);
 int set_error(int code, const char *fmt, ...);

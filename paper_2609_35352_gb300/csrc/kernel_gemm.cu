@@ -641,10 +641,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
 
 int gemm_configure(size_t smem)
 {
-    const cudaError_t e = cudaFuncSetAttribute((const void *)gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-    if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "matrix kernel attribute: %s", cudaGetErrorString(e));
-    return FIONA_OK;
+    return allow_shared_memory((const void *)gemm_kernel, smem, "matrix kernel attribute");
 }
 
 uint32_t gemm_units(const fiona_plan *p, uint32_t n_limbs)

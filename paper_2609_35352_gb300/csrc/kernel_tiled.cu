@@ -66,12 +66,9 @@ int tiled_kernel_attributes(int C, bool narrow, uint32_t P, bool kc, bool tc, cu
 int tiled_configure_kernel(int C, bool narrow, uint32_t P, bool kc, bool tc, size_t smem, bool off, bool w12,
                            bool ka)
 {
-    if (!select_ptr(C, narrow, P, kc, tc, off, w12, ka))
-        return set_error(FIONA_ERR_ARG, "tiled kernel: no variant with C=%d, P=%u", C, P);
-    cudaError_t e = cudaFuncSetAttribute(select_ptr(C, narrow, P, kc, tc, off, w12, ka),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "tiled kernel attribute: %s", cudaGetErrorString(e));
-    return FIONA_OK;
+    const void *fn = select_ptr(C, narrow, P, kc, tc, off, w12, ka);
+    if (!fn) return set_error(FIONA_ERR_ARG, "tiled kernel: no variant with C=%d, P=%u", C, P);
+    return allow_shared_memory(fn, smem, "tiled kernel attribute");
 }
 
 namespace {

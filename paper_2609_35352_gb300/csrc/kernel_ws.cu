@@ -394,9 +394,7 @@ int ws_configure_kernel(bool narrow, uint32_t P, bool kc, uint32_t W, uint32_t D
 {
     void *fn = select_ws(narrow, P, kc, W, D);
     if (!fn) return set_error(FIONA_ERR_ARG, "warp-specialised kernel: no variant with P=%u", P);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "ws kernel attribute: %s", cudaGetErrorString(e));
-    return FIONA_OK;
+    return allow_shared_memory(fn, smem, "ws kernel attribute");
 }
 
 // kernel_tiled.cu
