@@ -78,9 +78,10 @@ typedef enum fiona_status {
  * into shared memory (bulk asynchronous copies), shared signed sums are
  * formed once per tile, and the warps split the outputs.  AUTO (the default
  * after fiona_plan_create): DIRECT for a single output, for layers whose tile
- * does not fit in shared memory and for those a model of both kernels' time
- * puts at least a tenth quicker there (mostly few operands an output), TILED
- * otherwise.  For a layer whose every raw
+ * does not fit in shared memory and for launches that a model of both kernels'
+ * time puts well below there (few operands an output, or few limbs), TILED
+ * otherwise; the choice goes by the limbs of each launch, and the plan's
+ * statistics give the one for all of them.  For a layer whose every raw
  * plaintext is constant, TILED is the matrix kernel where the layer is large
  * enough for it (tile_coeffs 128: 128 coefficients of one poly per CTA, both
  * routes as exact products on the tensor cores). */

@@ -583,62 +583,94 @@ static int lower_tiled_optional(fiona_plan *p)
     return FIONA_OK;
 }
 
-// Whether a launch of `n_limbs` limbs takes the matrix kernel
-static bool use_gemm(const fiona_plan *p, uint32_t n_limbs)
+// Cycles of the direct kernel's longest output: its operations one after the
+// other, each waiting for its loads.
+static double direct_chain(const HostPlan &hp)
 {
-    return p->kernel == 1 && p->gemm && gemm_units(p, n_limbs) >= p->gemm->min_units;
+    double longest = 0;
+    std::vector<uint32_t> seen(hp.n_groups, 0);  // output + 1
+    for (uint32_t j = 0; j < hp.n_out; ++j) {
+        double c = 0;
+        for (uint32_t e = hp.term_offsets[j]; e < hp.term_offsets[j + 1]; ++e) {
+            const fiona_term &t = hp.terms[e];
+            if (t.kind != FIONA_TERM_TERNARY) {
+                c += 775;
+            } else if (t.sign != 0) {
+                c += 590;
+                if (seen[t.group] != j + 1) c += 960;
+                seen[t.group] = j + 1;
+            }
+        }
+        longest = std::max(longest, c);
+    }
+    return longest;
 }
 
-// Whether the direct kernel is expected to take at least 10% less time than the
-// tiled one: layers of few operands an output, where the tile (staging, padded
-// batches, one barrier) costs more than repeated reads through L2, and
-// launches too small to fill the tiled kernel's CTAs.  The direct kernel's time
-// is a sum over a coefficient's raw terms, signed terms, outputs, scale groups
-// and bytes, longer where few CTAs share the SMs (fitted on GB300 to 1391 random
-// layers of 3 to 150 inputs and 2 to 100 outputs: 5% from the measured time, one
-// standard deviation); of the 80 of 695 such layers where the rule takes it,
-// none ran longer and the mean was 0.80 of the tiled kernel's time.  Launches
-// below 16 us go by the operands an output has, six at most (3 -> 7 at 2^13 and
-// 5 limbs 10.9 us against 17.1; not two outputs, 4 -> 2 10.9 against 8.8), and by
-// the batches of four that scale groups of one term open (the smallest layer, 16
-// of them: 8.2 us against 10.2).
-static bool few_operands(const fiona_plan *p)
+// Whether a launch of `n_limbs` limbs is expected to be shorter on the direct
+// kernel than on the tiled one: layers of few operands an output, where the
+// tile (staging, padded batches, one barrier) costs more than repeated reads
+// through L2, and launches too small to fill the tiled kernel's CTAs.
+// The direct kernel's time joins its work (raw terms, signed terms, outputs,
+// scale groups and bytes, over the SMs) and its longest output by a norm; the
+// tiled kernel's is the shape model's, whose constant for a launch is of larger
+// ones (17000 cycles; small ones take 9900).  Both are fitted on GB300 to 6668
+// random layers of 6 us to 2 ms (2 to 150 inputs, 2 to 100 outputs, one scale
+// group an output or one a term), to
+//   time(inputs and plaintexts in L2)^2/3 time(not in L2)^1/3:
+// out of L2 the dependent loads of a long output cost the direct kernel more
+// than the tile's staging costs the other, but the operands of a small layer
+// have mostly just been written.  One standard deviation from the measured
+// time: 7% (direct: 4% for outputs of few operands, 10 to 13% for those of 64
+// whose chain is a third of the work or more) and 9% (tiled), of which the steps
+// of 2 us that short launches come in are 5.  So it takes a lead of a twentieth,
+// up to a quarter for such outputs, less half a microsecond.
+// Of 5043 other layers it took 2882, at 0.72 of the tiled kernel's time on
+// average; 153 ran more than 3% longer than there, 8 more than 10% (at worst 24%).
+static bool direct_is_quicker(const fiona_plan *p, uint32_t n_limbs)
 {
     const fiona_plan_stats_t &s = p->stats;
-    if (p->tiled->est_cycles < 33000) {
-        const uint64_t terms = s.n_nonzero_terms;
-        return (p->hp.n_out > 2 && terms <= 6ull * p->hp.n_out) ||
-               (p->hp.n_in <= 8 && 2ull * std::max<uint64_t>(s.n_scale_groups_used, p->hp.n_out) >= terms);
-    }
     const double raw = s.n_raw_terms, groups = s.n_scale_groups_used, n_out = p->hp.n_out;
-    const double coeffs = (double)p->ctx->N * p->ctx->L, sms = p->ctx->sm_count > 0 ? p->ctx->sm_count : 152;
+    const double per_sm = (double)p->ctx->N * n_limbs / (p->ctx->sm_count > 0 ? p->ctx->sm_count : 152);
     const double bytes = (raw + groups + 2.0 * s.n_inputs_used + 2 * n_out) * 8;
-    const double each = 0.385 * raw + 0.294 * s.n_signed_terms + 1.4 * n_out + 0.27 * groups + bytes / 27.5;
-    const double ctas = coeffs / 256 * n_out;
-    const double cycles = 15400 + coeffs / sms * each * (1 + 0.28 * 16 * sms / ctas);
-    return cycles < 0.9 * p->tiled->est_cycles;
+    const double work = per_sm * (0.48 * raw + 0.32 * s.n_signed_terms + 1.03 * n_out + 0.55 * groups + bytes / 28.7);
+    const double direct = 10700 + std::pow(std::pow(work, 1.9) + std::pow(p->direct_chain, 1.9), 1 / 1.9);
+    const double tiled = p->tiled->est_cycles[n_limbs - 1] - 17000 + 9900;
+    const double lead =
+        0.05 + 0.2 * std::min(1.0, s.n_nonzero_terms / (64 * n_out)) * std::min(1.0, p->direct_chain / (0.3 * work));
+    return direct < (1 - lead) * tiled + 1000;
+}
+
+// Whether a launch of `n_limbs` limbs runs on the tiled kernel (or the matrix
+// kernel in its place)
+static bool takes_tiled(const fiona_plan *p, uint32_t n_limbs)
+{
+    if (!p->automatic) return p->kernel == 1;
+    if (!p->tiled || p->hp.n_out < 2) return false;
+    return p->shape_asked || !direct_is_quicker(p, n_limbs);
+}
+
+// Whether a launch of `n_limbs` limbs takes the matrix kernel
+static bool takes_gemm(const fiona_plan *p, uint32_t n_limbs)
+{
+    return p->gemm && (p->automatic || p->kernel == 1) && gemm_units(p, n_limbs) >= p->gemm->min_units;
 }
 
 // Kernel choice: DIRECT for a single output (no input reuse to exploit), where
-// the tile does not fit in shared memory, and for layers of few operands an
-// output, unless a shape of the tiled kernel is asked for; TILED otherwise
-// (every input is then read from HBM once).
+// the tile does not fit in shared memory, and for launches expected to be
+// quicker there (direct_is_quicker), unless a shape of the tiled kernel is asked
+// for; TILED otherwise (every input is then read from HBM once).
 static int select_kernel(fiona_plan *p, int which)
 {
-    int k;
-    if (which == FIONA_KERNEL_DIRECT)
-        k = 0;
-    else if (which == FIONA_KERNEL_TILED)
-        k = 1;
-    else if (which == FIONA_KERNEL_AUTO)
-        k = (p->tiled && p->hp.n_out > 1 && (p->shape_asked || p->gemm || !few_operands(p))) ? 1 : 0;
-    else
+    if (which != FIONA_KERNEL_DIRECT && which != FIONA_KERNEL_TILED && which != FIONA_KERNEL_AUTO)
         return set_error(FIONA_ERR_ARG, "select_kernel: unknown variant %d", which);
-    if (k == 1 && !p->tiled && p->ctx->device != FIONA_DEVICE_NONE)
+    if (which == FIONA_KERNEL_TILED && !p->tiled && p->ctx->device != FIONA_DEVICE_NONE)
         return set_error(FIONA_ERR_ARG, "select_kernel: the tiled kernel cannot run this plan");
+    p->automatic = which == FIONA_KERNEL_AUTO;
+    const uint32_t L = p->ctx->L;
+    const int k = p->automatic ? takes_gemm(p, L) || takes_tiled(p, L) : which == FIONA_KERNEL_TILED;
     p->kernel = k;
     fiona_plan_stats_t &s = p->stats;
-    if (use_gemm(p, p->ctx->L)) {
+    if (takes_gemm(p, L)) {
         s.kernel = FIONA_KERNEL_TILED;
         s.tile_coeffs = kGemmRows;
         s.warps_per_cta = kGemmThreads / 32;
@@ -756,6 +788,7 @@ extern "C" int fiona_plan_create(const fiona_ctx *ctx, uint32_t n_in, uint32_t n
         return rc;
     }
     compute_stats(ctx, hp, p->stats);
+    p->direct_chain = direct_chain(hp);
     // lazy-reduction budgets from the largest modulus
     const u128 qm1 = ctx->q_max - 1;
     const u128 mb = (~(u128)0) / (qm1 * qm1);
@@ -891,8 +924,8 @@ static int check_eval_args(const fiona_plan *p, const void *in, const void *pt, 
 static int launch_range(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt,
                         uint64_t *out, uint32_t l0, uint32_t l1, uint32_t layout_L)
 {
-    if (use_gemm(p, l1 - l0)) return launch_gemm(p, stream, in, pt, out, l0, l1, layout_L);
-    if (p->kernel == 1) return launch_tiled(p, stream, in, pt, out, l0, l1, layout_L);
+    if (takes_gemm(p, l1 - l0)) return launch_gemm(p, stream, in, pt, out, l0, l1, layout_L);
+    if (takes_tiled(p, l1 - l0)) return launch_tiled(p, stream, in, pt, out, l0, l1, layout_L);
     return launch_direct(p, stream, in, pt, out, l0, l1, layout_L);
 }
 

@@ -74,7 +74,9 @@ struct fiona_plan {
     fiona_plan_stats_t stats{};
     uint32_t mac_budget = 0;     // products a 128-bit accumulator may take before a reduction
     uint32_t signed_budget = 0;  // residues a 64-bit signed accumulator may take
-    int kernel = 0;              // 0 = direct, 1 = tiled (what evaluations use)
+    int kernel = 0;              // 0 = direct, 1 = tiled (launches over every limb)
+    bool automatic = true;       // the kernel goes by each launch's limbs
+    double direct_chain = 0;     // cycles of the direct kernel's longest output
     bool shape_asked = false;    // a tuning override named a shape of the tiled kernel
     // direct schedule (device pointers into sched.blob)
     DeviceSchedule sched;

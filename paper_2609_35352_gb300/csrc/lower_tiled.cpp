@@ -1704,7 +1704,7 @@ int lower_tiled(fiona_plan *p)
         double balance = 0;           // mean warp cost / largest warp cost
         uint32_t keep = 0, ctas = 0;  // shared sums requested (top of the ranking)
         size_t smem = 0;
-        std::vector<double> level;    // predicted cycles at all limbs, one less, ... half of them
+        std::vector<double> level;    // predicted cycles at one limb, two, ... all of them
     };
     // plans with constant plaintexts run the kernel variant that reads them
     bool has_const = false;
@@ -1809,7 +1809,7 @@ int lower_tiled(fiona_plan *p)
                 s.keep = hi;
                 s.ctas = ctas;
                 s.smem = smem - attr.sharedSizeBytes;
-                for (uint32_t n = ctx->L; 2 * n >= ctx->L && n; --n)
+                for (uint32_t n = 1; n <= ctx->L; ++n)
                     s.level.push_back(
                         model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W, deepest,
                                      (prods + 2.0 * hp.n_in + 2.0 * hp.n_out) * T * 8, hp.n_in, jp.n_part, s.smem,
@@ -1819,7 +1819,7 @@ int lower_tiled(fiona_plan *p)
                     fprintf(stderr,
                             "C=%d P=%u W=%u dbl=%d w12=%d keep=%u sched=%zu parts=%u smem=%zu ctas=%u pad=%.2f est=%.0f\n",
                             C, batch, W, (int)dbl, (int)w12, s.keep, sc.w.size() * 4, jp.n_part, smem, ctas, s.pad,
-                            s.level[0]);
+                            s.level.back());
             }
         }
     }
@@ -1843,7 +1843,7 @@ int lower_tiled(fiona_plan *p)
         const bool deep = s.w12 && s.W == 12 && s.P == 8 && s.balance >= 0.95;
         const int pref = s.C == 2 ? (deep ? 3 : s.P == 4 ? 2 : 1) : (s.P == 16 ? 2 : s.P == 8 ? 1 : 0);
         const uint32_t resident = deep ? 16 : std::min<uint32_t>(s.ctas * s.W, 16);
-        return std::make_tuple(s.dbl ? 1 : 0, resident, s.C, s.ctas, pref, -s.level[0]);
+        return std::make_tuple(s.dbl ? 1 : 0, resident, s.C, s.ctas, pref, -s.level.back());
     };
     Shape best = *std::max_element(shapes.begin(), shapes.end(),
                                    [&](const Shape &a, const Shape &b) { return key(a) < key(b); });
@@ -1863,11 +1863,11 @@ int lower_tiled(fiona_plan *p)
     const double margin = hp.n_out < 8 ? 0.75 : narrow ? 0.86 : 0.88;
     const Shape *quick = nullptr;
     for (const Shape &a : shapes) {
-        bool ok = a.level[0] < margin * best.level[0];
-        for (size_t i = 1; i < a.level.size(); ++i) ok &= a.level[i] <= 1.03 * best.level[i];
-        if (ok && (!quick || a.level[0] < quick->level[0])) quick = &a;
+        bool ok = a.level.back() < margin * best.level.back();
+        for (size_t n = (ctx->L + 1) / 2; n < ctx->L; ++n) ok &= a.level[n - 1] <= 1.03 * best.level[n - 1];
+        if (ok && (!quick || a.level.back() < quick->level.back())) quick = &a;
     }
-    if (!p->shape_asked && best.level[0] > 82800 && quick) best = Shape(*quick);
+    if (!p->shape_asked && best.level.back() > 82800 && quick) best = Shape(*quick);
     // tuning override "C,W,double[,most shared sums kept[,P]]": every shape
     // computes the same residues
     if (const char *env = getenv("FIONA_TILED_SHAPE")) {
@@ -2082,7 +2082,7 @@ int lower_tiled(fiona_plan *p)
     ts->warps = best.W;
     ts->tile = T;
     ts->batch = best.P;
-    ts->est_cycles = best.level[0];
+    ts->est_cycles = best.level;
     ts->has_const = has_const;
     ts->smem = best.smem;
     ts->ctas_per_sm = best.ctas;

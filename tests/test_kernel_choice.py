@@ -1,9 +1,8 @@
 """Which kernel and shape a plan takes by itself (FIONA_KERNEL_AUTO), on both
-sides of the rule's lines: the direct kernel where the model of its time is a
-tenth below the tiled kernel's, and for small launches of few operands an
-output, unless a shape of the tiled kernel is asked for; the tiled kernel's shape
-where the model of its time moves it.  Every choice gives the same residues (GPU
-parity)."""
+sides of the rule's lines: the direct kernel where the model of its time is far
+enough below the tiled kernel's, unless a shape of the tiled kernel is asked for;
+the tiled kernel's shape where the model of its time moves it.  Every choice
+gives the same residues (GPU parity)."""
 import pytest
 
 from paper_2609_35352_gb300 import build as B
@@ -26,7 +25,7 @@ def stats(n_in, n_out, N=1 << 16, L=4, bits=50, signed=0.5, per_term=False, desc
 @pytest.mark.parametrize("n_in,n_out,L,bits,signed,direct", [
     (3, 49, 4, 60, 0.54, True), (3, 73, 10, 40, 0.0, False),     # three operands an output: wide, narrow
     (4, 9, 13, 45, 0.95, True), (6, 65, 2, 50, 0.1, False),
-    (113, 9, 5, 60, 1.0, True), (112, 4, 3, 60, 0.9, False),     # many inputs, few outputs
+    (112, 3, 3, 60, 0.9, True), (112, 4, 3, 60, 0.9, False),     # many inputs, few outputs
     (64, 1, 4, 50, 0.5, True),                                   # one output
 ])
 def test_direct_kernel(n_in, n_out, L, bits, signed, direct):
@@ -34,16 +33,35 @@ def test_direct_kernel(n_in, n_out, L, bits, signed, direct):
     assert k == (F.FIONA_KERNEL_DIRECT if direct else F.FIONA_KERNEL_TILED)
 
 
-def test_small_launches_and_overrides(monkeypatch):
-    small = dict(N=4096, L=3)
-    assert stats(6, 6, **small)["kernel"] == F.FIONA_KERNEL_DIRECT    # six operands an output
-    assert stats(7, 6, **small)["kernel"] == F.FIONA_KERNEL_TILED
-    assert stats(4, 2, **small)["kernel"] == F.FIONA_KERNEL_TILED     # two outputs
-    assert stats(8, 4, **small)["kernel"] == F.FIONA_KERNEL_TILED
-    wl = W.make_workload("tiny")  # a batch of four per one-term group
+# at N = 2^12 and 3 limbs, the inputs up to which a layer of n outputs is direct:
+# one group a term (a batch of four each on the tiled kernel), one group an output
+SMALL = {(True, 50): {2: 4, 3: 7, 4: 9, 6: 16}, (False, 50): {3: 4, 4: 6, 6: 8, 8: 8, 12: 12, 16: 14},
+         (False, 60): {2: 7, 3: 8, 4: 8, 6: 16, 8: 16, 12: 24}}
+
+
+@pytest.mark.parametrize("per_term,bits,n_out", [(*k, n) for k, v in SMALL.items() for n in v])
+def test_small_launches(per_term, bits, n_out):
+    """One line in the inputs, direct below it and tiled above, which moves up
+    with the outputs, the modulus and the groups."""
+    line = SMALL[per_term, bits][n_out]
+    got = [stats(n_in, n_out, N=4096, L=3, bits=bits, per_term=per_term)["kernel"] == F.FIONA_KERNEL_DIRECT
+           for n_in in (line // 2, max(line * 2 // 3, 2), line * 4 // 3 + 1, line * 2 + 2)]
+    assert got == [True, True, False, False], got
+
+
+@pytest.mark.parametrize("n_in,n_out,N,bits,few,many", [(16, 16, 2048, 50, 2, 6), (24, 24, 4096, 50, 1, 6),
+                                                        (7, 7, 65536, 50, 1, 8), (11, 11, 65536, 60, 1, 8)])
+def test_fewer_limbs(n_in, n_out, N, bits, few, many):
+    """The choice goes by the limbs of a launch: direct for few of them."""
+    assert stats(n_in, n_out, N=N, L=few, bits=bits)["kernel"] == F.FIONA_KERNEL_DIRECT
+    assert stats(n_in, n_out, N=N, L=many, bits=bits)["kernel"] == F.FIONA_KERNEL_TILED
+
+
+def test_smallest_layer_and_overrides(monkeypatch):
+    wl = W.make_workload("tiny")
     assert stats(8, 4, N=wl.N, L=wl.L, bits=40, desc=wl.plan)["kernel"] == F.FIONA_KERNEL_DIRECT
     monkeypatch.setenv("FIONA_TILED_SHAPE", "2,4,1")
-    assert stats(6, 6, **small)["kernel"] == F.FIONA_KERNEL_TILED
+    assert stats(6, 6, N=4096, L=3)["kernel"] == F.FIONA_KERNEL_TILED
 
 
 def test_tiled_shape():
