@@ -25,7 +25,7 @@
 //      operations a slot at 2^15 slots (a butterfly six, or four additions
 //      where the twiddle is 1 or -i) against 66 with the negacyclic
 //      Gentleman-Sande stages before, whose butterflies take eight.  Measured
-//      on GB300, 93 vectors of 2^15 slots: 0.435 -> 0.324 ms.
+//      on GB300, 93 vectors of 2^15 slots: 0.435 -> 0.326 ms.
 //   2. RNS/NTT form: c_i mod q_l for every limb, then the forward NTT mod
 //      q_l (ntt.cuh, the tables the rescale uses), canonical.
 // Step 1 is floating point: it reproduces round(Delta m_i) except where

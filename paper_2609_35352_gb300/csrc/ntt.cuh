@@ -197,10 +197,13 @@ struct CplxArith {
         x = make_double2(re, im);
     }
     // x - w y on its own, eight operations: one rounding less.  Taken in the last
-    // stage of each pass, which brings the transform's error just below that of
-    // the eight-operation stages before (relative 2-norm at 2^15 slots, measured
-    // against 113-bit arithmetic: 2.75e-16 against 2.78e-16, without it 2.80e-16;
-    // embedding 93 vectors 0.324 ms against 0.315)
+    // stage of each pass, and from 2^15 slots on in the last two of the high
+    // pass: the transform's error is then below that of eight-operation stages
+    // throughout at every ring size (relative 2-norm against extended precision,
+    // complex slots: 2.11e-16 against 2.20e-16 at 2^9, 2.70 against 2.71 at 2^14,
+    // 2.79 against 2.81 at 2^15, 2.875 against 2.887 at 2^16; with one stage only
+    // 2.896 there).  Embedding 93 vectors of 2^15: 0.326 ms, 0.322 with one
+    // stage, 0.315 with none.
     __device__ __forceinline__ static void butterfly_direct(T &x, T &y, W w)
     {
         const double2 a = x, b = y;
@@ -346,6 +349,8 @@ __device__ __forceinline__ void cyclic_stages(typename A::T (&x)[1 << PS::K(R)],
                                               const typename A::Staged &stw)
 {
     constexpr int K = PS::K(R), LD = Group<PS, R>::LD;
+    // the last stages of the pass by direct butterflies (CplxArith)
+    constexpr int direct = PS::high && PS::s + PS::lsubs + PS::ltiles >= 15 ? 2 : 1;
 #pragma unroll
     for (int t = 0; t < K; ++t)
 #pragma unroll
@@ -360,7 +365,7 @@ __device__ __forceinline__ void cyclic_stages(typename A::T (&x)[1 << PS::K(R)],
                     A::butterfly_1(x[b], x[b + (1 << t)]);
                 else if (minus_i)
                     A::butterfly_i(x[b], x[b + (1 << t)]);
-                else if (R == 0 && t == K - 1)
+                else if (R == 0 && t >= K - direct)
                     A::butterfly_direct(x[b], x[b + (1 << t)], w);
                 else
                     A::butterfly(x[b], x[b + (1 << t)], w);
