@@ -83,6 +83,33 @@ def test_matrix_kernel_parity(n_in, n_out, share, N, bits, L, fill, monkeypatch)
     assert dl.ctx.device_check() == F.FIONA_OK
 
 
+@pytest.mark.parametrize("n_in,n_out,bits", [
+    (17, 17, (50, 34, 45, 40)),       # one step and a half of 16 inputs, a block with one group
+    (33, 49, (34, 50, 42, 50)),       # an odd number of steps, a last block with one group
+    (81, 200, (49, 36, 50)),          # two chunks of outputs: 128 and 72
+])
+def test_matrix_kernel_walk(n_in, n_out, bits, monkeypatch):
+    """Several units a CTA, whose ranges cross limbs (of moduli of different
+    widths: the digits and biases are made again) and chunks (other outputs):
+    every barrier's parity, the unit's coordinates and the next unit's
+    prefetches, counted on from unit to unit."""
+    monkeypatch.setenv("FIONA_CONST_GEMM", "1")
+    N = 8192
+    moduli = [W.ntt_primes(N, b, 1 + i)[i] for i, b in enumerate(bits)]
+    plan, n_raw = layer(n_in, n_out, 0.5, 7 * n_in)
+    wl = W.Workload("gemm", N, moduli, plan, 31 + n_in, const_pts=n_raw)
+    dl = DeviceLayer(wl)
+    dl.plan.select_kernel("tiled")
+    assert dl.plan.stats()["tile_coeffs"] == 128
+    units = (2 if n_out > 128 else 1) * len(moduli) * (N // 128) * 2
+    assert units > 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    dl.run()
+    want = oracle.linear_eval(plan, wl.moduli, dl.X, dl.P)
+    mism = np.argwhere(dl.outputs() != want)
+    assert mism.shape[0] == 0, "first mismatches (j, c, l, k): %s of %d" % (mism[:5].tolist(), mism.shape[0])
+    assert dl.ctx.device_check() == F.FIONA_OK
+
+
 def test_matrix_kernel_extreme_digits(monkeypatch):
     """Weights and residues around 0, q / 2 and the digit boundaries, whose
     centred digits are the largest; 64 raw terms in every output."""
