@@ -164,11 +164,12 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_enc_high(EncArgs
 }
 
 // RNS/NTT form, forward low stages, canonical store: the same rows of kPolys
-// polys per CTA (blockIdx.x = (group * Lc + limb) * tiles + tile)
-template <int LOGN, bool FAST>
-__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 4) k_enc_low(EncArgs A)
+// polys per CTA, or of one (many_polys; blockIdx.x = (group * Lc + limb) * tiles
+// + tile)
+template <int LOGN, bool FAST, int LP>
+__global__ void __launch_bounds__(LowPassPolys<LOGN, LP>::threads, LP ? 4 : 12) k_enc_low(EncArgs A)
 {
-    using PS = LowPassPolys<LOGN>;
+    using PS = LowPassPolys<LOGN, LP>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), tr = blockIdx.x >> PS::ltiles;
     const uint32_t p0 = (tr / A.Lc) << PS::lpolys, l = tr % A.Lc;
@@ -268,17 +269,18 @@ template <int LOGN>
 struct Inst {
     static constexpr size_t emb_low = LowPass<LOGN - 1>::template smem_bytes<CplxArith>();
     static constexpr size_t emb_high = HighPass<LOGN - 1>::template smem_bytes<CplxArith>();
+    static constexpr size_t enc_low1 = LowPassPolys<LOGN, 0>::template smem_bytes<ModArith<false>>();
     static constexpr size_t enc_low = LowPassPolys<LOGN>::template smem_bytes<ModArith<false>>();
     static constexpr size_t enc_high = HighPass<LOGN>::template smem_bytes<ModArith<false>>();
 };
 
 struct Kernels {
     EmbKern emb_low, emb_high;
-    EncKern enc_high[2], enc_low[2];
-    size_t s_emb_low, s_emb_high, s_enc_high, s_enc_low;
+    EncKern enc_high[2], enc_low[2][2];  // by FAST; low pass: one poly a CTA, kPolys
+    size_t s_emb_low, s_emb_high, s_enc_high, s_enc_low[2];
     // log2 tiles per transform and threads per CTA of each pass
     uint32_t lt_emb_low, lt_emb_high, lt_enc_high, lt_enc_low;
-    uint32_t t_emb_low, t_emb_high, t_enc_high, t_enc_low;
+    uint32_t t_emb_low, t_emb_high, t_enc_high, t_enc_low[2];
 };
 
 template <int LOGN>
@@ -287,11 +289,12 @@ constexpr Kernels kernels_for()
     return Kernels{k_embed_low<LOGN - 1>,
                    k_embed_high<LOGN - 1>,
                    {k_enc_high<LOGN, false>, k_enc_high<LOGN, true>},
-                   {k_enc_low<LOGN, false>, k_enc_low<LOGN, true>},
+                   {{k_enc_low<LOGN, false, 0>, k_enc_low<LOGN, false, kLogPolys>},
+                    {k_enc_low<LOGN, true, 0>, k_enc_low<LOGN, true, kLogPolys>}},
                    Inst<LOGN>::emb_low,
                    Inst<LOGN>::emb_high,
                    Inst<LOGN>::enc_high,
-                   Inst<LOGN>::enc_low,
+                   {Inst<LOGN>::enc_low1, Inst<LOGN>::enc_low},
                    LowPass<LOGN - 1>::ltiles,
                    HighPass<LOGN - 1>::ltiles,
                    HighPass<LOGN>::ltiles,
@@ -299,7 +302,7 @@ constexpr Kernels kernels_for()
                    LowPass<LOGN - 1>::threads,
                    HighPass<LOGN - 1>::threads,
                    HighPass<LOGN>::threads,
-                   LowPassPolys<LOGN>::threads};
+                   {LowPassPolys<LOGN, 0>::threads, LowPassPolys<LOGN>::threads}};
 }
 
 const Kernels &kernels(uint32_t n)
@@ -321,7 +324,8 @@ int configure(const fiona_ctx *ctx, uint32_t n)
     const std::pair<const void *, size_t> fs[] = {
         {(const void *)K.emb_low, K.s_emb_low},         {(const void *)K.emb_high, K.s_emb_high},
         {(const void *)K.enc_high[0], K.s_enc_high},    {(const void *)K.enc_high[1], K.s_enc_high},
-        {(const void *)K.enc_low[0], K.s_enc_low},      {(const void *)K.enc_low[1], K.s_enc_low}};
+        {(const void *)K.enc_low[0][0], K.s_enc_low[0]}, {(const void *)K.enc_low[1][0], K.s_enc_low[0]},
+        {(const void *)K.enc_low[0][1], K.s_enc_low[1]}, {(const void *)K.enc_low[1][1], K.s_enc_low[1]}};
     for (const auto &f : fs) {
         const cudaError_t e = cudaFuncSetAttribute(f.first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.second);
         if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "encode: kernel attributes: %s", cudaGetErrorString(e));
@@ -395,9 +399,10 @@ int launch_encode_coeffs(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64
         a.coeffs = coeffs + p0 * ctx->N;
         a.out = out + p0 * Lc * (uint64_t)ctx->N;
         a.count = (uint32_t)np;
-        const uint64_t nt = np * Lc, ng = (np + kPolys - 1) / kPolys;
+        const int many = many_polys(ctx, np, Lc);
+        const uint64_t nt = np * Lc, ng = many ? (np + kPolys - 1) / kPolys : np;
         K.enc_high[fast]<<<(uint32_t)(nt << K.lt_enc_high), K.t_enc_high, K.s_enc_high, s>>>(a);
-        K.enc_low[fast]<<<(uint32_t)((ng * Lc) << K.lt_enc_low), K.t_enc_low, K.s_enc_low, s>>>(a);
+        K.enc_low[fast][many]<<<(uint32_t)((ng * Lc) << K.lt_enc_low), K.t_enc_low[many], K.s_enc_low[many], s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "encode launch: %s", cudaGetErrorString(e));

@@ -139,6 +139,9 @@ void free_rescale_tables(const fiona_ctx *ctx);
 namespace fiona_ntt {
 struct NttLimb;
 }
+// whether a low pass over `count` polys of `limbs` limbs takes eight polys a CTA
+// rather than one
+bool many_polys(const fiona_ctx *ctx, uint64_t count, uint32_t limbs);
 // the modular NTT tables of every limb (built on the first call)
 int ntt_tables(const fiona_ctx *ctx, const fiona_ntt::NttLimb **limbs);
 

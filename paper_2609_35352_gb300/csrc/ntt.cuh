@@ -22,8 +22,9 @@
 //              a CTA takes tile / R2 blocks.
 // A CTA's tile is 4096 elements in the high pass; in the low pass, whose CTAs
 // also stage about one twiddle per element, it is the same rows of eight polys
-// (4096 elements, 512 twiddles) for the transforms mod q and 2048 elements of
-// one for the complex ones.  A thread handles 16 elements.
+// (4096 elements, 512 twiddles) for the transforms mod q, or of one poly where
+// there are few, and 2048 elements of one for the complex ones.  A thread
+// handles 16 elements (8 of a tile of 512).
 // A pass runs its stages in rounds of up to 4: in a round each thread holds
 // the 2^K elements of one group in registers, spaced by the round's smallest
 // distance, and applies the round's K stages to them (a group needs 2^K - 1
@@ -286,9 +287,10 @@ using LowPass = PassShape<LowShape<LOGN>::s, LowShape<LOGN>::lt - LowShape<LOGN>
 // (45 KB a CTA of 256 threads).  Measured on GB300, 192 polys of 2^16, 12
 // limbs: the rescale 1.488 ms with 4 polys a CTA, 1.410 with 8.
 constexpr int kLogPolys = 3, kPolys = 1 << kLogPolys;
-template <int LOGN>
-using LowPassPolys = PassShape<LOGN - Shape<LOGN>::n1, kLogTileMax - (LOGN - Shape<LOGN>::n1), false,
-                               LOGN - kLogTileMax + kLogPolys, kLogPolys>;
+// LP = kLogPolys, or fewer polys with the same rows (and the same table)
+template <int LOGN, int LP = kLogPolys>
+using LowPassPolys = PassShape<LOGN - Shape<LOGN>::n1, kLogTileMax - (LOGN - Shape<LOGN>::n1) - kLogPolys + LP, false,
+                               LOGN - kLogTileMax + kLogPolys, LP>;
 
 // Group g of round R: sub-transform `sub`, and the element positions
 // (hi << (lD + K)) + (i << lD) + lo, i < 2^K.  High pass: sub-transforms

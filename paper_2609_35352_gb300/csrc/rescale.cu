@@ -56,14 +56,15 @@ struct Args {
 // The four launches.  blockIdx.x = transform * tiles + tile; the transforms
 // are the polys (inverse high pass), poly * (Lc - 1) + limb (forward high
 // pass), and for the low passes, whose CTAs take the same rows of kPolys
-// polys, group of polys (inverse) or group * (Lc - 1) + limb (forward).
+// polys or of one (many_polys), group of polys (inverse) or group * (Lc - 1) +
+// limb (forward).
 // ---------------------------------------------------------------------------
 
 // inverse, low stages, on the last limb in place
-template <int LOGN>
-__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 3) k_inv_low(Args A)
+template <int LOGN, int LP>
+__global__ void __launch_bounds__(LowPassPolys<LOGN, LP>::threads, LP ? 3 : 12) k_inv_low(Args A)
 {
-    using PS = LowPassPolys<LOGN>;
+    using PS = LowPassPolys<LOGN, LP>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), p0 = (blockIdx.x >> PS::ltiles) << PS::lpolys;
     const uint32_t first = tile << PS::lrows;
@@ -128,10 +129,10 @@ __global__ void __launch_bounds__(HighPass<LOGN>::threads, 3) k_fwd_high(Args A)
 }
 
 // forward, low stages, then y' = (y_l - t) * q_{Lc-1}^-1
-template <int LOGN, bool FAST>
-__global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 3) k_fwd_low(Args A)
+template <int LOGN, bool FAST, int LP>
+__global__ void __launch_bounds__(LowPassPolys<LOGN, LP>::threads, LP ? 3 : 12) k_fwd_low(Args A)
 {
-    using PS = LowPassPolys<LOGN>;
+    using PS = LowPassPolys<LOGN, LP>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t tile = blockIdx.x & ((1u << PS::ltiles) - 1), tr = blockIdx.x >> PS::ltiles;
     const uint32_t p0 = (tr / (A.Lc - 1)) << PS::lpolys, l = tr % (A.Lc - 1);
@@ -166,6 +167,44 @@ __global__ void __launch_bounds__(LowPassPolys<LOGN>::threads, 3) k_fwd_low(Args
                         canon6(mul_twiddle(v + M - t_of(e0, t), qi, q), q);
                 });
         });
+}
+
+typedef void (*Kern)(Args);
+
+// A ring dimension's launches; the low passes with one poly a CTA and with kPolys
+struct Kernels {
+    Kern inv_low[2], inv_high, fwd_high[2], fwd_low[2][2];
+    // log2 tiles per transform, threads and shared memory per CTA
+    uint32_t lt_low, lt_high, t_low[2], t_high;
+    size_t s_low[2], s_high;
+};
+
+template <int LOGN>
+constexpr Kernels kernels_for()
+{
+    typedef ModArith<false> MA;
+    using Low1 = LowPassPolys<LOGN, 0>;
+    using Low = LowPassPolys<LOGN>;
+    using High = HighPass<LOGN>;
+    static_assert((int)Low1::ltiles == (int)Low::ltiles, "the same tiles");
+    return Kernels{{k_inv_low<LOGN, 0>, k_inv_low<LOGN, kLogPolys>},
+                   k_inv_high<LOGN>,
+                   {k_fwd_high<LOGN, false>, k_fwd_high<LOGN, true>},
+                   {{k_fwd_low<LOGN, false, 0>, k_fwd_low<LOGN, false, kLogPolys>},
+                    {k_fwd_low<LOGN, true, 0>, k_fwd_low<LOGN, true, kLogPolys>}},
+                   Low::ltiles,
+                   High::ltiles,
+                   {Low1::threads, Low::threads},
+                   High::threads,
+                   {Low1::template smem_bytes<MA>(), Low::template smem_bytes<MA>()},
+                   High::template smem_bytes<MA>()};
+}
+
+const Kernels &kernels(uint32_t n)
+{
+    static const Kernels K[] = {kernels_for<10>(), kernels_for<11>(), kernels_for<12>(), kernels_for<13>(),
+                                kernels_for<14>(), kernels_for<15>(), kernels_for<16>(), kernels_for<17>()};
+    return K[n - kLogNMin];
 }
 
 // ---------------------------------------------------------------------------
@@ -304,6 +343,23 @@ int ntt_tables(const fiona_ctx *ctx, const fiona_ntt::NttLimb **limbs)
     return rc;
 }
 
+// One poly a CTA (64 threads) where those CTAs are few, up to `per_sm` an SM: a
+// CTA of eight polys takes longer and leaves more of the GPU idle; and where the
+// groups of eight are mostly absent polys, up to `few` of eight.  Both by the
+// measured times: the one-poly CTAs of 2^7 and 2^8 positions idle half their
+// threads in rounds of four stages.  GB300, rescale of 12 limbs, one poly against
+// eight a CTA: 2^16, one poly 35.0 us against 44.3, two 47.3 - 50.4, three 56.5 -
+// 53.6; 2^17, one 43.3 - 76.0, four 96.5 - 107.7, eight 171.5 - 163.2; 2^14, four
+// 31.0 - 32.9, sixteen 53.4 - 49.4; 2^10, any count to 32 18.6 - 24.8.
+bool many_polys(const fiona_ctx *ctx, uint64_t count, uint32_t limbs)
+{
+    const uint32_t n = log2u(ctx->N), s = n - n / 2;
+    const uint64_t ctas = count * ((uint64_t)limbs << (n - kLogTileMax + kLogPolys));
+    const uint64_t groups = (count + kPolys - 1) / kPolys;
+    const uint64_t few = s == 8 ? 2 : s == 7 ? 4 : 5, per_sm = s == 8 ? 2 : s == 7 ? 5 : 13;
+    return ctas > per_sm * std::max(ctx->sm_count, 1) && count > few * groups;
+}
+
 int launch_rescale(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64_t count, uint64_t *polys, uint64_t *out,
                    bool round)
 {
@@ -319,59 +375,32 @@ int launch_rescale(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64_t cou
     const uint64_t qlast = ctx->moduli[Lc - 1];
     for (uint32_t l = 0; l + 1 < Lc; ++l)
         if (ctx->moduli[l] >= (1ull << 56) || qlast >= 4 * ctx->moduli[l]) fast = false;
-    const int ix = (int)n - kLogNMin;
-    typedef void (*Kern)(Args);
-    static const Kern inv_low[] = {k_inv_low<10>, k_inv_low<11>, k_inv_low<12>, k_inv_low<13>,
-                                   k_inv_low<14>, k_inv_low<15>, k_inv_low<16>, k_inv_low<17>};
-    static const Kern inv_high[] = {k_inv_high<10>, k_inv_high<11>, k_inv_high<12>, k_inv_high<13>,
-                                    k_inv_high<14>, k_inv_high<15>, k_inv_high<16>, k_inv_high<17>};
-    static const Kern fwd_high[2][8] = {
-        {k_fwd_high<10, false>, k_fwd_high<11, false>, k_fwd_high<12, false>, k_fwd_high<13, false>,
-         k_fwd_high<14, false>, k_fwd_high<15, false>, k_fwd_high<16, false>, k_fwd_high<17, false>},
-        {k_fwd_high<10, true>, k_fwd_high<11, true>, k_fwd_high<12, true>, k_fwd_high<13, true>,
-         k_fwd_high<14, true>, k_fwd_high<15, true>, k_fwd_high<16, true>, k_fwd_high<17, true>}};
-    static const Kern fwd_low[2][8] = {
-        {k_fwd_low<10, false>, k_fwd_low<11, false>, k_fwd_low<12, false>, k_fwd_low<13, false>,
-         k_fwd_low<14, false>, k_fwd_low<15, false>, k_fwd_low<16, false>, k_fwd_low<17, false>},
-        {k_fwd_low<10, true>, k_fwd_low<11, true>, k_fwd_low<12, true>, k_fwd_low<13, true>,
-         k_fwd_low<14, true>, k_fwd_low<15, true>, k_fwd_low<16, true>, k_fwd_low<17, true>}};
-    // per pass: tiles per transform (log2) and threads per CTA
-#define FIONA_GEO(P) {P<10>::ltiles, P<11>::ltiles, P<12>::ltiles, P<13>::ltiles, P<14>::ltiles, P<15>::ltiles, P<16>::ltiles, P<17>::ltiles}
-#define FIONA_THR(P) {P<10>::threads, P<11>::threads, P<12>::threads, P<13>::threads, P<14>::threads, P<15>::threads, P<16>::threads, P<17>::threads}
-    static const int low_lt[] = FIONA_GEO(LowPassPolys), high_lt[] = FIONA_GEO(HighPass);
-    static const uint32_t low_thr[] = FIONA_THR(LowPassPolys), high_thr[] = FIONA_THR(HighPass);
-#undef FIONA_GEO
-#undef FIONA_THR
-    const uint32_t lt_low = (uint32_t)low_lt[ix], lt_high = (uint32_t)high_lt[ix];
-    const Kern ks[4] = {inv_low[ix], inv_high[ix], fwd_high[fast][ix], fwd_low[fast][ix]};
-    typedef ModArith<false> MA;
-    static const size_t low_smem[] = {
-        LowPassPolys<10>::smem_bytes<MA>(), LowPassPolys<11>::smem_bytes<MA>(), LowPassPolys<12>::smem_bytes<MA>(),
-        LowPassPolys<13>::smem_bytes<MA>(), LowPassPolys<14>::smem_bytes<MA>(), LowPassPolys<15>::smem_bytes<MA>(),
-        LowPassPolys<16>::smem_bytes<MA>(), LowPassPolys<17>::smem_bytes<MA>()};
-    static const size_t high_smem[] = {
-        HighPass<10>::smem_bytes<MA>(), HighPass<11>::smem_bytes<MA>(), HighPass<12>::smem_bytes<MA>(),
-        HighPass<13>::smem_bytes<MA>(), HighPass<14>::smem_bytes<MA>(), HighPass<15>::smem_bytes<MA>(),
-        HighPass<16>::smem_bytes<MA>(), HighPass<17>::smem_bytes<MA>()};
-    const size_t smem[4] = {low_smem[ix], high_smem[ix], high_smem[ix], low_smem[ix]};
+    const Kernels &K = kernels(n);
     cudaError_t e = cudaSuccess;
     {
-        // the dynamic shared memory limit, once per device and kernel
-        static bool configured[FIONA_MAX_DEVICES][kLogNMax - kLogNMin + 1][2] = {};
+        // the dynamic shared memory limits, once per device and ring dimension
+        static bool configured[FIONA_MAX_DEVICES][kLogNMax - kLogNMin + 1] = {};
         std::lock_guard<std::mutex> lock(g_ntt_mu);
         if (ctx->device < 0 || ctx->device >= FIONA_MAX_DEVICES)
             return set_error(FIONA_ERR_ARG, "rescale: device %d", ctx->device);
-        if (!configured[ctx->device][ix][fast]) {
-            for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-                e = cudaFuncSetAttribute((const void *)ks[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem[i]);
+        if (!configured[ctx->device][n - kLogNMin]) {
+            auto limit = [&](Kern k, size_t bytes) {
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            };
+            limit(K.inv_high, K.s_high);
+            for (int f = 0; f < 2; ++f) limit(K.fwd_high[f], K.s_high);
+            for (int m = 0; m < 2; ++m) {
+                limit(K.inv_low[m], K.s_low[m]);
+                for (int f = 0; f < 2; ++f) limit(K.fwd_low[f][m], K.s_low[m]);
+            }
             if (e != cudaSuccess)
                 return set_error(FIONA_ERR_CUDA, "rescale: kernel attributes: %s", cudaGetErrorString(e));
-            configured[ctx->device][ix][fast] = true;
+            configured[ctx->device][n - kLogNMin] = true;
         }
     }
     // grid.x < 2^31: transforms * tiles, in chunks of whole polys
-    const uint64_t max_polys = ((1ull << 31) - 1) / ((uint64_t)(Lc - 1) << std::max(lt_low, lt_high));
+    const uint64_t max_polys = ((1ull << 31) - 1) / ((uint64_t)(Lc - 1) << std::max(K.lt_low, K.lt_high));
     cudaStream_t s = (cudaStream_t)stream;
     for (uint64_t p0 = 0; p0 < count && e == cudaSuccess; p0 += max_polys) {
         const uint64_t np = std::min<uint64_t>(count - p0, max_polys);
@@ -382,11 +411,13 @@ int launch_rescale(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64_t cou
         a.count = (uint32_t)np;
         a.Lc = Lc;
         a.round = round ? 1 : 0;
-        const uint64_t nf = np * (Lc - 1), ng = (np + kPolys - 1) / kPolys;
-        ks[0]<<<(uint32_t)(ng << lt_low), low_thr[ix], smem[0], s>>>(a);
-        ks[1]<<<(uint32_t)(np << lt_high), high_thr[ix], smem[1], s>>>(a);
-        ks[2]<<<(uint32_t)(nf << lt_high), high_thr[ix], smem[2], s>>>(a);
-        ks[3]<<<(uint32_t)((ng * (Lc - 1)) << lt_low), low_thr[ix], smem[3], s>>>(a);
+        const uint64_t nf = np * (Lc - 1);
+        const int mi = many_polys(ctx, np, 1), mf = many_polys(ctx, np, Lc - 1);
+        const uint64_t gi = mi ? (np + kPolys - 1) / kPolys : np, gf = mf ? (np + kPolys - 1) / kPolys : np;
+        K.inv_low[mi]<<<(uint32_t)(gi << K.lt_low), K.t_low[mi], K.s_low[mi], s>>>(a);
+        K.inv_high<<<(uint32_t)(np << K.lt_high), K.t_high, K.s_high, s>>>(a);
+        K.fwd_high[fast]<<<(uint32_t)(nf << K.lt_high), K.t_high, K.s_high, s>>>(a);
+        K.fwd_low[fast][mf]<<<(uint32_t)((gf * (Lc - 1)) << K.lt_low), K.t_low[mf], K.s_low[mf], s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return set_error(FIONA_ERR_CUDA, "rescale launch: %s", cudaGetErrorString(e));

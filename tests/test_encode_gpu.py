@@ -146,7 +146,10 @@ def random_coeffs(seed, count, N):
 
 
 @pytest.mark.parametrize("N,L,bits,count", [(1024, 3, 50, 3), (2048, 2, 60, 2), (8192, 3, 40, 2),
-                                            (65536, 12, 50, 2), (131072, 2, 59, 1)])
+                                            (65536, 12, 50, 2), (131072, 2, 59, 1),
+                                            # eight polys a CTA, the last group of three
+                                            (1024, 2, 50, 1003), (4096, 2, 60, 251), (16384, 2, 45, 67),
+                                            (65536, 2, 50, 19), (131072, 2, 50, 11)])
 def test_encode_coeffs_parity(N, L, bits, count):
     qs = W.ntt_primes(N, bits, L)
     ctx = F.Context(N, qs, device=0)

@@ -243,11 +243,25 @@ def test_layer_and_rescale_replay_in_a_cuda_graph(shape, tile, monkeypatch):
         assert np.array_equal(to_host(out).reshape(p.n_out * 2, wl.L - 1, wl.N), want)
 
 
+# polys from which the low passes of one limb take eight a CTA, with an incomplete group
+MANY = [(1024, 50, 1003), (4096, 60, 251), (16384, 45, 67), (65536, 50, 19), (131072, 50, 11)]
+
+
+@pytest.mark.parametrize("N,bits,count", MANY)
+def test_many_polys(N, bits, count):
+    """The low passes take the same rows of eight polys per CTA: whole and
+    incomplete groups, rows of 32 to 512 elements."""
+    qs = W.ntt_primes(N, bits, 2)
+    y = random_polys(19 * count, qs, count, N)
+    ctx = F.Context(N, qs, device=0)
+    got, _ = gpu_rescale(ctx, y, 2)
+    assert np.array_equal(got, oracle.rescale(qs, y))
+
+
 @pytest.mark.parametrize("count", [1, 7, 8, 11])
 @pytest.mark.parametrize("N,bits", [(1024, 50), (4096, 60), (16384, 45), (131072, 50)])
 def test_groups_of_polys(N, bits, count):
-    """The low passes take the same rows of eight polys per CTA: whole and
-    incomplete groups, rows of 32 to 512 elements."""
+    """Few polys: one per CTA of the low passes (at 2^17, some groups of eight)."""
     qs = W.ntt_primes(N, bits, 3)
     y = random_polys(17 * count, qs, count, N)
     ctx = F.Context(N, qs, device=0)
