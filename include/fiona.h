@@ -82,9 +82,10 @@ typedef enum fiona_status {
  * time puts well below there (few operands an output, or few limbs), TILED
  * otherwise; the choice goes by the limbs of each launch, and the plan's
  * statistics give the one for all of them.  For a layer whose every raw
- * plaintext is constant, TILED is the matrix kernel where the layer is large
- * enough for it (tile_coeffs 128: 128 coefficients of one poly per CTA, both
- * routes as exact products on the tensor cores). */
+ * plaintext is constant, launches that it is quicker for run on the matrix
+ * kernel in TILED's place (statistics: kernel TILED, tile_coeffs 128: 128
+ * coefficients of one poly per CTA, both routes as exact products on the tensor
+ * cores). */
 enum { FIONA_KERNEL_AUTO = 0, FIONA_KERNEL_DIRECT = 1, FIONA_KERNEL_TILED = 2 };
 
 /* Pass as `device` to fiona_ctx_create for a validation-only context: plans

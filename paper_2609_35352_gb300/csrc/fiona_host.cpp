@@ -606,10 +606,11 @@ static double direct_chain(const HostPlan &hp)
     return longest;
 }
 
-// Whether a launch of `n_limbs` limbs is expected to be shorter on the direct
-// kernel than on the tiled one: layers of few operands an output, where the
-// tile (staging, padded batches, one barrier) costs more than repeated reads
-// through L2, and launches too small to fill the tiled kernel's CTAs.
+// Predicted SM cycles of a launch of `n_limbs` limbs on the tiled and on the
+// direct kernel, and whether the direct one leads by enough to take it: layers of
+// few operands an output, where the tile (staging, padded batches, one barrier)
+// costs more than repeated reads through L2, and launches too small to fill the
+// tiled kernel's CTAs.
 // The direct kernel's time joins its work (raw terms, signed terms, outputs,
 // scale groups and bytes, over the SMs) and its longest output by a norm; the
 // tiled kernel's is the shape model's, whose constant for a launch is of larger
@@ -626,7 +627,12 @@ static double direct_chain(const HostPlan &hp)
 // up to a quarter for such outputs, less half a microsecond.
 // Of 5043 other layers it took 2882, at 0.72 of the tiled kernel's time on
 // average; 153 ran more than 3% longer than there, 8 more than 10% (at worst 24%).
-static bool direct_is_quicker(const fiona_plan *p, uint32_t n_limbs)
+struct LaunchCycles {
+    double tiled, direct;
+    bool direct_leads;
+};
+
+static LaunchCycles launch_cycles(const fiona_plan *p, uint32_t n_limbs)
 {
     const fiona_plan_stats_t &s = p->stats;
     const double raw = s.n_raw_terms, groups = s.n_scale_groups_used, n_out = p->hp.n_out;
@@ -637,40 +643,45 @@ static bool direct_is_quicker(const fiona_plan *p, uint32_t n_limbs)
     const double tiled = p->tiled->est_cycles[n_limbs - 1] - 17000 + 9900;
     const double lead =
         0.05 + 0.2 * std::min(1.0, s.n_nonzero_terms / (64 * n_out)) * std::min(1.0, p->direct_chain / (0.3 * work));
-    return direct < (1 - lead) * tiled + 1000;
+    return {tiled, direct, direct < (1 - lead) * tiled + 1000};
 }
 
-// Whether a launch of `n_limbs` limbs runs on the tiled kernel (or the matrix
-// kernel in its place)
-static bool takes_tiled(const fiona_plan *p, uint32_t n_limbs)
+// The matrix kernel runs a launch that it is a microsecond quicker for, by the
+// models, than the kernel that would run it otherwise (GB300, 1455 random layers:
+// 355 take it, at 0.70 of that kernel's time on average; 6 run 3 to 9% longer).
+static bool matrix_leads(const fiona_plan *p, uint32_t n_limbs, double other)
 {
-    if (!p->automatic) return p->kernel == 1;
-    if (!p->tiled || p->hp.n_out < 2) return false;
-    return p->shape_asked || !direct_is_quicker(p, n_limbs);
+    return p->gemm && (p->gemm->always || gemm_cycles(p, n_limbs) + 2000 < other);
 }
 
-// Whether a launch of `n_limbs` limbs takes the matrix kernel
-static bool takes_gemm(const fiona_plan *p, uint32_t n_limbs)
+// Kernel choice for launches of `n_limbs` limbs.  AUTO: direct for a single
+// output (no input reuse to exploit), where the tile does not fit in shared
+// memory, and for launches expected to be quicker there (launch_cycles), unless a
+// shape of the tiled kernel is asked for; tiled otherwise (every input is then
+// read from HBM once); the matrix kernel in the place of either, or of the tiled
+// one where that is asked for.
+static Route route_for(const fiona_plan *p, int which, uint32_t n_limbs)
 {
-    return p->gemm && (p->automatic || p->kernel == 1) && gemm_units(p, n_limbs) >= p->gemm->min_units;
+    const bool may_tile = p->tiled && (which == FIONA_KERNEL_TILED || p->hp.n_out > 1);
+    if (which == FIONA_KERNEL_DIRECT || !may_tile)
+        return which == FIONA_KERNEL_TILED ? Route::tiled : Route::direct;
+    if (p->shape_asked) return matrix_leads(p, n_limbs, 0) ? Route::matrix : Route::tiled;
+    const LaunchCycles c = launch_cycles(p, n_limbs);
+    const bool direct = which == FIONA_KERNEL_AUTO && c.direct_leads;
+    if (matrix_leads(p, n_limbs, direct ? c.direct : c.tiled)) return Route::matrix;
+    return direct ? Route::direct : Route::tiled;
 }
 
-// Kernel choice: DIRECT for a single output (no input reuse to exploit), where
-// the tile does not fit in shared memory, and for launches expected to be
-// quicker there (direct_is_quicker), unless a shape of the tiled kernel is asked
-// for; TILED otherwise (every input is then read from HBM once).
 static int select_kernel(fiona_plan *p, int which)
 {
     if (which != FIONA_KERNEL_DIRECT && which != FIONA_KERNEL_TILED && which != FIONA_KERNEL_AUTO)
         return set_error(FIONA_ERR_ARG, "select_kernel: unknown variant %d", which);
     if (which == FIONA_KERNEL_TILED && !p->tiled && p->ctx->device != FIONA_DEVICE_NONE)
         return set_error(FIONA_ERR_ARG, "select_kernel: the tiled kernel cannot run this plan");
-    p->automatic = which == FIONA_KERNEL_AUTO;
-    const uint32_t L = p->ctx->L;
-    const int k = p->automatic ? takes_gemm(p, L) || takes_tiled(p, L) : which == FIONA_KERNEL_TILED;
-    p->kernel = k;
+    for (uint32_t n = 1; n <= p->ctx->L; ++n) p->route[n - 1] = route_for(p, which, n);
+    const Route r = p->route[p->ctx->L - 1];
     fiona_plan_stats_t &s = p->stats;
-    if (takes_gemm(p, L)) {
+    if (r == Route::matrix) {
         s.kernel = FIONA_KERNEL_TILED;
         s.tile_coeffs = kGemmRows;
         s.warps_per_cta = kGemmThreads / 32;
@@ -681,7 +692,7 @@ static int select_kernel(fiona_plan *p, int which)
         s.tensor_core_sums = p->gemm->groups;
         s.source_offsets = 0;
         s.const_raw_all = 1;
-    } else if (k == 1 && p->tiled) {
+    } else if (r == Route::tiled && p->tiled) {
         s.kernel = FIONA_KERNEL_TILED;
         s.tile_coeffs = p->tiled->tile;
         s.warps_per_cta = p->tiled->warps;
@@ -924,9 +935,11 @@ static int check_eval_args(const fiona_plan *p, const void *in, const void *pt, 
 static int launch_range(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt,
                         uint64_t *out, uint32_t l0, uint32_t l1, uint32_t layout_L)
 {
-    if (takes_gemm(p, l1 - l0)) return launch_gemm(p, stream, in, pt, out, l0, l1, layout_L);
-    if (takes_tiled(p, l1 - l0)) return launch_tiled(p, stream, in, pt, out, l0, l1, layout_L);
-    return launch_direct(p, stream, in, pt, out, l0, l1, layout_L);
+    switch (p->route[l1 - l0 - 1]) {
+    case Route::matrix: return launch_gemm(p, stream, in, pt, out, l0, l1, layout_L);
+    case Route::tiled: return launch_tiled(p, stream, in, pt, out, l0, l1, layout_L);
+    default: return launch_direct(p, stream, in, pt, out, l0, l1, layout_L);
+    }
 }
 
 extern "C" int fiona_linear_eval(const fiona_plan *p, void *stream, const uint64_t *in,

@@ -68,14 +68,15 @@ struct HostPlan {
     std::vector<int32_t> term_use;  // use index covering term e, or -1
 };
 
+enum class Route : uint8_t { direct, tiled, matrix };
+
 struct fiona_plan {
     const fiona_ctx *ctx = nullptr;
     HostPlan hp;
     fiona_plan_stats_t stats{};
     uint32_t mac_budget = 0;     // products a 128-bit accumulator may take before a reduction
     uint32_t signed_budget = 0;  // residues a 64-bit signed accumulator may take
-    int kernel = 0;              // 0 = direct, 1 = tiled (launches over every limb)
-    bool automatic = true;       // the kernel goes by each launch's limbs
+    Route route[FIONA_MAX_LIMBS] = {};  // the kernel of launches over 1, 2, ... all limbs
     double direct_chain = 0;     // cycles of the direct kernel's longest output
     bool shape_asked = false;    // a tuning override named a shape of the tiled kernel
     // direct schedule (device pointers into sched.blob)
@@ -87,8 +88,8 @@ struct fiona_plan {
     const uint32_t *d_raw_pt = nullptr;
     // tiled schedule
     TiledSchedule *tiled = nullptr;
-    // matrix kernel's schedule, where it can run the layer and pays: the
-    // tiled variant of such a plan for launches of enough units
+    // matrix kernel's schedule, where it can run the layer: in the place of
+    // the other kernels for launches that it is quicker for
     GemmSchedule *gemm = nullptr;
     // streams for fiona_linear_eval_host(_async), and per limb chunk the
     // events of its last input copy, kernel and output copy: a call orders
@@ -128,6 +129,7 @@ int launch_tiled(const fiona_plan *p, void *stream, const uint64_t *in, const ui
 int lower_gemm(fiona_plan *p);
 void free_gemm(fiona_plan *p);
 uint32_t gemm_units(const fiona_plan *p, uint32_t n_limbs);
+double gemm_cycles(const fiona_plan *p, uint32_t n_limbs);
 int launch_gemm(const fiona_plan *p, void *stream, const uint64_t *in, const uint64_t *pt, uint64_t *out,
                 uint32_t limb_begin, uint32_t limb_end, uint32_t layout_L);
 

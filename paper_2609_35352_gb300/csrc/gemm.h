@@ -102,5 +102,5 @@ struct GemmSchedule {
     size_t smem = 0;
     DeviceSchedule sched;
     uint32_t groups = 0;      // scale groups
-    uint32_t min_units = 0;   // units of a launch from which this kernel runs
+    bool always = false;      // runs whatever its predicted time
 };

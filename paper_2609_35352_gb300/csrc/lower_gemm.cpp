@@ -1,5 +1,5 @@
 // lower_gemm.cpp -- lowering of a layer whose raw plaintexts are all constant
-// to the matrix kernel's schedule (gemm.h), and the rule that picks it.
+// to the matrix kernel's schedule (gemm.h), and the model of that kernel's time.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -16,20 +16,26 @@ namespace {
 // the most dynamic shared memory a CTA may have (227 KB)
 constexpr size_t kSmemMax = 232448;
 
-// Cycles of a warp scheduler per 32 coefficients of both polys, fitted to both
-// kernels on GB300 (layers of 8 to 96 inputs and outputs, a quarter to three
-// quarters raw, N = 2^12 to 2^16).  At 16 x 16 with 144 products (128 raw terms
-// and 16 gammas) the matrix kernel measured 1.08-1.19 times faster, with 80 it
-// was even (0.91-1.00), at 8 x 8 it took 1.7-2 times as long, at 96 x 96 a
-// third to a quarter.
-double tiled_cost(uint64_t products, uint64_t signed_terms) { return 3500.0 + 30.0 * products + 6.0 * signed_terms; }
-double gemm_cost(uint32_t n_in, uint32_t n_out) { return 4000.0 + 3400.0 * ((n_out + 15) / 16) + 52.0 * n_in; }
-
 }  // namespace
 
-// Builds p->gemm where the matrix kernel can run the layer and is expected to
-// be faster; leaves it null otherwise.  FIONA_CONST_GEMM=0 never builds it, =1
-// whenever it can run (and for launches of any size).
+// Predicted SM cycles of a launch over `n_limbs` limbs: the making of G's digits,
+// and the units of the CTA that has most, each by its blocks of 32 outputs,
+// groups of 16 and inputs (fitted on GB300 to 1455 random layers of 2 to 96
+// inputs and 2 to 100 outputs, N = 2^10 to 2^16, 1 to 12 limbs, 10 us to 2 ms, to
+// the scale of the other kernels' models: 4% from the measured time, one standard
+// deviation)
+double gemm_cycles(const fiona_plan *p, uint32_t n_limbs)
+{
+    const GemmArgs &a = p->gemm->args;
+    const uint32_t units = gemm_units(p, n_limbs), sms = p->ctx->sm_count > 0 ? p->ctx->sm_count : 152;
+    const double chunks = a.n_chunks, groups = (a.n_out + 15) / 16 / chunks;
+    const double blocks = (a.n_out + kGemmBlock - 1) / kGemmBlock / chunks;
+    const double unit = 2130 + 1700 * blocks + (2450 + 12.4 * a.K) * groups + 47.0 * a.K;
+    return 16400 + 9.5 * p->stats.n_raw_terms / chunks + (units + sms - 1) / sms * unit;
+}
+
+// Builds p->gemm where the matrix kernel can run the layer; leaves it null
+// otherwise.  FIONA_CONST_GEMM=0 never builds it; =1 has it run whatever its time.
 int lower_gemm(fiona_plan *p)
 {
     const HostPlan &hp = p->hp;
@@ -68,7 +74,6 @@ int lower_gemm(fiona_plan *p)
         sgn_row.push_back((uint32_t)sgn.size());
     }
     if (raw.empty()) return FIONA_OK;
-    if (!force && tiled_cost(raw.size() + groups.size(), sgn.size()) < gemm_cost(hp.n_in, hp.n_out)) return FIONA_OK;
 
     const uint32_t K = (hp.n_in + 15) & ~15u, blocks = (hp.n_out + kGemmBlock - 1) / kGemmBlock;
     uint32_t fit = blocks;  // blocks of outputs per CTA
@@ -83,10 +88,7 @@ int lower_gemm(fiona_plan *p)
     GemmSchedule *g = new GemmSchedule;
     g->smem = GemmLayout(K, chunk).total;
     g->groups = (uint32_t)groups.size();
-    // below one unit per SM, too few CTAs share the work (each also makes G's
-    // digits) and the tiled kernel runs; measured at 192 units (N = 2^12, 3
-    // limbs): even at 16 x 16, 1.2 times faster at 32 x 24
-    g->min_units = force ? 0 : std::max(ctx->sm_count, 1);
+    g->always = force;
     GemmArgs &a = g->args;
     a.limbs = ctx->d_limbs;
     a.err = ctx->d_kerr;

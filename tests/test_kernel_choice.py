@@ -57,6 +57,19 @@ def test_fewer_limbs(n_in, n_out, N, bits, few, many):
     assert stats(n_in, n_out, N=N, L=many, bits=bits)["kernel"] == F.FIONA_KERNEL_TILED
 
 
+@pytest.mark.parametrize("n_in,n_out,N,L,signed,matrix", [
+    (96, 96, 1 << 16, 12, 0.53, True), (80, 17, 1 << 15, 2, 0.9, True),
+    (12, 91, 1 << 15, 2, 0.5, True), (12, 91, 1 << 15, 1, 0.5, True), (12, 91, 1 << 11, 1, 0.5, False),
+    (16, 10, 1 << 14, 2, 0.0, False), (19, 11, 1 << 15, 6, 0.3, False), (8, 8, 1 << 16, 12, 0.5, False),
+])
+def test_matrix_kernel(n_in, n_out, N, L, signed, matrix):
+    """Constant raw plaintexts: the matrix kernel (128 coefficients a unit) where
+    its time leads those of both others."""
+    tern = int(n_in * n_out * signed)
+    desc = W.constant_raw_plan(W.dense_hybrid_plan(W.PlanRng(7), n_in, n_out, tern // 2, tern // 2, 0))
+    assert (stats(0, 0, N=N, L=L, desc=desc)["tile_coeffs"] == 128) == matrix
+
+
 def test_smallest_layer_and_overrides(monkeypatch):
     wl = W.make_workload("tiny")
     assert stats(8, 4, N=wl.N, L=wl.L, bits=40, desc=wl.plan)["kernel"] == F.FIONA_KERNEL_DIRECT
