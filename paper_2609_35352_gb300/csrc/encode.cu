@@ -383,7 +383,8 @@ int launch_encode_coeffs(const fiona_ctx *ctx, void *stream, uint32_t Lc, uint64
     if (rc == FIONA_OK) rc = configure(ctx, n);
     if (rc) return rc;
     if (count == 0) return FIONA_OK;
-    // the reduction-free butterflies need every q_l < 2^56 (inputs are canonical)
+    // the reduction-free butterflies need every q_l < 2^56 and inputs below 8 q_l,
+    // as k_enc_high loads them
     bool fast = true;
     for (uint32_t l = 0; l < Lc; ++l)
         if (ctx->moduli[l] >= (1ull << 56)) fast = false;

@@ -613,8 +613,9 @@ static double direct_chain(const HostPlan &hp)
 // tiled kernel's CTAs.
 // The direct kernel's time joins its work (raw terms, signed terms, outputs,
 // scale groups and bytes, over the SMs) and its longest output by a norm; the
-// tiled kernel's is the shape model's, whose constant for a launch is of larger
-// ones (17000 cycles; small ones take 9900).  Both are fitted on GB300 to 6668
+// tiled kernel's is the shape model's, with a last round of few CTAs at their own
+// time and the constant of small launches (9900 cycles; the model's 17000 is of
+// larger ones).  Both are fitted on GB300 to 6668
 // random layers of 6 us to 2 ms (2 to 150 inputs, 2 to 100 outputs, one scale
 // group an output or one a term), to
 //   time(inputs and plaintexts in L2)^2/3 time(not in L2)^1/3:
@@ -622,11 +623,12 @@ static double direct_chain(const HostPlan &hp)
 // than the tile's staging costs the other, but the operands of a small layer
 // have mostly just been written.  One standard deviation from the measured
 // time: 7% (direct: 4% for outputs of few operands, 10 to 13% for those of 64
-// whose chain is a third of the work or more) and 9% (tiled), of which the steps
-// of 2 us that short launches come in are 5.  So it takes a lead of a twentieth,
-// up to a quarter for such outputs, less half a microsecond.
-// Of 5043 other layers it took 2882, at 0.72 of the tiled kernel's time on
-// average; 153 ran more than 3% longer than there, 8 more than 10% (at worst 24%).
+// whose chain is a third of the work or more) and 8% (tiled), of which the steps
+// of 2 us that short launches come in are 5.  So it takes a lead of 3%, up to
+// 23% for such outputs, less 0.7 us.
+// Of 5043 other layers it took 3040, at 0.73 of the tiled kernel's time on
+// average; 204 ran more than 3% longer than there (mostly out of L2), 10 more than
+// 10% (at worst 32%).
 struct LaunchCycles {
     double tiled, direct;
     bool direct_leads;
@@ -642,13 +644,14 @@ static LaunchCycles launch_cycles(const fiona_plan *p, uint32_t n_limbs)
     const double direct = 10700 + std::pow(std::pow(work, 1.9) + std::pow(p->direct_chain, 1.9), 1 / 1.9);
     const double tiled = p->tiled->est_cycles[n_limbs - 1] - 17000 + 9900;
     const double lead =
-        0.05 + 0.2 * std::min(1.0, s.n_nonzero_terms / (64 * n_out)) * std::min(1.0, p->direct_chain / (0.3 * work));
-    return {tiled, direct, direct < (1 - lead) * tiled + 1000};
+        0.03 + 0.2 * std::min(1.0, s.n_nonzero_terms / (64 * n_out)) * std::min(1.0, p->direct_chain / (0.3 * work));
+    return {tiled, direct, direct < (1 - lead) * tiled + 1500};
 }
 
 // The matrix kernel runs a launch that it is a microsecond quicker for, by the
 // models, than the kernel that would run it otherwise (GB300, 1455 random layers:
-// 355 take it, at 0.70 of that kernel's time on average; 6 run 3 to 9% longer).
+// 343 take it, at 0.70 of that kernel's time on average; 3 run 3 to 9% longer; of
+// 1471 others 353, at 0.69, 12 of them 3 to 20% longer).
 static bool matrix_leads(const fiona_plan *p, uint32_t n_limbs, double other)
 {
     return p->gemm && (p->gemm->always || gemm_cycles(p, n_limbs) + 2000 < other);

@@ -24,18 +24,13 @@
 // and 108 of N = 32 at the 50 cycles each needs whatever N <= 96) run under
 // them but for each unit's first block.  Measured on GB300 (96 -> 96 outputs,
 // 4332 constant raw terms, 12 limbs of 2^16): 5.383 ms on the tiled kernel,
-// whose products keep the FMA-heavy pipe busy; here 4.33 ms with the issue
-// loops not unrolled, 2.02 unrolled, 1.59 with uniform control flow in the
-// issuing warp and the recombination in words, 1.44 with the digit weights
-// read at run time, 1.29 with the signed sums in shared memory, counted unit
-// coordinates and the shorter quotient.  The layer's 3.0 GB take 0.45 ms.
-// Starting a unit's multiplications when the first third of its digits is
-// there took it from 1.290 to 1.280; leaving the waits as whole warps, to 1.288
-// (below).  Making the next unit's digits under the
-// last group's epilogue (1.44), 112 registers a worker by setmaxnreg (1.32),
-// prefetching gamma's tiles to L1 (no change), the products by gamma formed
-// with the signed sums (1.31) and additions and shifts in place of some of the
-// recombination's multiplications (1.285 to 1.288) were not kept.
+// whose products keep the FMA-heavy pipe busy, 1.288 here; the layer's 3.0 GB
+// take 0.45 ms.  Each of these made it slower: rolled issue loops (4.3 ms),
+// lane-dependent control flow in the issuing warp and 128-bit arithmetic in the
+// recombination (2.0), literal digit weights (1.6), the signed sums in registers
+// (1.44), the next unit's digits under the last group's epilogue (1.44), 112
+// registers a worker by setmaxnreg, the products by gamma formed with the signed
+// sums (both 2%).
 // All waits are bounded (GemmArgs::wait_ns on the global timer); one that
 // gives up sets the context's error flag and the CTA's abort flag, which ends
 // every other wait; each warp then stops as a whole, at the end of its unit or
@@ -216,7 +211,10 @@ __host__ __device__ constexpr uint64_t magic_sum(int n)
 }
 
 // Per output: the bias of the raw sum, cut into the parts of weights 1, 2^32
-// and 2^64 (each at least what makes that part of the sum positive)
+// and 2^64.  With theirs the words of weights 1 and 2^32 are not negative; b2,
+// and the word of weight 2^64 with it, is negative for narrow moduli (t is about
+// 2^74 at 34 bits, less 2^18 borrowed here): that word counts modulo 2^64, and the
+// sum of the three modulo 2^128, where it is the true one, in [0, 2^(2k+9)).
 struct __align__(16) OutBias {
     uint64_t b0, b1, b2, pad;
 };
@@ -606,7 +604,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const GemmArgs a)
                     for (uint32_t i = 0; i < 4; ++i) {
                         const OutBias b = bias[o1 + i];
                         // the classes as three words of weights 1, 2^32, 2^64,
-                        // each with its part of the bias: none is negative
+                        // each with its part of the bias (OutBias)
                         uint64_t l0 = b.b0 + magic(e[0][i]);
                         l0 = mad_wide(magic(e[1][i]), a.c8, l0);
                         l0 = mad_wide(magic(e[2][i]), a.c16, l0);

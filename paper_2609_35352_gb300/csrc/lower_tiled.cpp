@@ -120,27 +120,36 @@ struct ShapeModel {
     double hbm;                // bytes a cycle
     double launch;             // a launch
 
-    // rounds of tiles over the SMs: a launch of few tiles leaves CTA slots empty
+    // rounds of tiles over the SMs: a launch of few tiles leaves CTA slots empty.
+    // `tail`: a last round of at most half the CTAs an SM at their own time, 8.0%
+    // from the measured times of 11.5 k launches where the whole round is 9.3%, up
+    // to a quarter too long when it is nearly empty.  (The shapes are compared by whole
+    // rounds, as the margins below were tuned.)
     double cycles(int C, uint32_t W, uint32_t P, bool dbl, uint32_t ctas, double demand, double longest, double deepest,
-                  double bytes, uint32_t n_in, uint32_t n_part, size_t smem, double tiles_per_sm) const
+                  double bytes, uint32_t n_in, uint32_t n_part, size_t smem, double tiles_per_sm, bool tail) const
     {
         // what the shared memory leaves of the SM's 256 KB for the L1
         uint32_t carve = 228;
         for (uint32_t kb : {196u, 164u, 132u, 100u, 64u, 32u, 16u, 8u})
             if ((double)ctas * ((double)smem + 1088) <= kb * 1024.0) carve = kb;
         const double l1 = (256.0 - carve) * 1024;
-        const double live = std::min((double)ctas, std::ceil(tiles_per_sm));
-        const double flight = live * W * P * 32 * C * 8;
-        const double terms[4] = {live * demand / 4, longest * c[C - 1].latency, live * bytes / hbm,
-                                 deepest / P * fetch * std::max(1.0, flight / (window * l1))};
-        double t = 0;
-        for (double x : terms) t += std::pow(x, norm);
-        t = std::pow(t, 1 / norm);
-        const double in = (double)n_in * C;
-        t += ((dbl ? ahead + ahead_in * in : stage + stage_in * in) + part * n_part) * (live == 1 ? 1.0 : share);
-        if (C == 2 && W == 16 && P == 8) t *= 1.1;  // (register spills)
-        const double rounds = tiles_per_sm / live;
-        return t * (rounds < 4 ? std::ceil(rounds) : rounds + 0.4) + launch;
+        // a round of tiles with `live` CTAs on the SM
+        auto round = [&](double live) {
+            const double flight = live * W * P * 32 * C * 8;
+            const double terms[4] = {live * demand / 4, longest * c[C - 1].latency, live * bytes / hbm,
+                                     deepest / P * fetch * std::max(1.0, flight / (window * l1))};
+            double t = 0;
+            for (double x : terms) t += std::pow(x, norm);
+            t = std::pow(t, 1 / norm);
+            const double in = (double)n_in * C;
+            t += ((dbl ? ahead + ahead_in * in : stage + stage_in * in) + part * n_part) * (live == 1 ? 1.0 : share);
+            if (C == 2 && W == 16 && P == 8) t *= 1.1;  // (register spills)
+            return t;
+        };
+        const double live = std::min((double)ctas, std::ceil(tiles_per_sm)), rounds = tiles_per_sm / live;
+        if (!tail) return round(live) * (rounds < 4 ? std::ceil(rounds) : rounds + 0.4) + launch;
+        const double whole = std::floor(rounds + 1e-9), rest = tiles_per_sm - whole * live;
+        return whole * round(live) + (rest > 1e-6 ? round(2 * rest <= live ? std::ceil(rest) : live) : 0) + launch;
     }
 };
 const ShapeModel kNarrowModel{{{41.8, 13.6, 235, 229, 1.44}, {50.6, 21.1, 415, 329, 1.86}},
@@ -1705,6 +1714,7 @@ int lower_tiled(fiona_plan *p)
         uint32_t keep = 0, ctas = 0;  // shared sums requested (top of the ranking)
         size_t smem = 0;
         std::vector<double> level;    // predicted cycles at one limb, two, ... all of them
+        std::vector<double> launch;   // the same, a last round of fewer CTAs at their own time
     };
     // plans with constant plaintexts run the kernel variant that reads them
     bool has_const = false;
@@ -1810,10 +1820,12 @@ int lower_tiled(fiona_plan *p)
                 s.ctas = ctas;
                 s.smem = smem - attr.sharedSizeBytes;
                 for (uint32_t n = 1; n <= ctx->L; ++n)
-                    s.level.push_back(
-                        model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W, deepest,
-                                     (prods + 2.0 * hp.n_in + 2.0 * hp.n_out) * T * 8, hp.n_in, jp.n_part, s.smem,
-                                     (double)ctx->N / T * n / (double)sms));
+                    for (bool tail : {false, true})
+                        (tail ? s.launch : s.level)
+                            .push_back(model.cycles(C, W, batch, dbl, ctas, demand + node_ops, longest + node_ops / W,
+                                                    deepest, (prods + 2.0 * hp.n_in + 2.0 * hp.n_out) * T * 8,
+                                                    hp.n_in, jp.n_part, s.smem, (double)ctx->N / T * n / (double)sms,
+                                                    tail));
                 shapes.push_back(s);
                 if (getenv("FIONA_TILED_DEBUG"))
                     fprintf(stderr,
@@ -1848,14 +1860,14 @@ int lower_tiled(fiona_plan *p)
     Shape best = *std::max_element(shapes.begin(), shapes.end(),
                                    [&](const Shape &a, const Shape &b) { return key(a) < key(b); });
     // Away from the layers that ranking was made on, the shape the model puts
-    // first, where it promises more than 1.65 times a prediction's error (14%, and
-    // 12% with wide moduli; with 12% for both one layer in 600, 11 -> 63 of 50
-    // bits at 2^13, became 5% slower; 25% below eight outputs, whose split work
-    // it knows less well) and
-    // the launch takes at least 40 us.  On 778 random layers (2^15, up to 8
-    // limbs) it moved the time per layer by 4 to 6% on average, at best 100
-    // inputs -> 40 outputs: 1.96 ms with one coefficient per lane, two regions and
-    // 2 x 8 warps, 0.91 with two and one region; at worst 4% up.
+    // first, where it promises 14% (12% with wide moduli, 25% below eight outputs,
+    // whose split work it knows less well) and the launch takes at least 40 us.
+    // The margins are tuned: about 1.65 standard deviations of a prediction, then
+    // the narrow one raised from 12% for one layer in 600 (11 -> 63 of 50 bits at
+    // 2^13) that had become 5% slower.  On 778 random layers (2^15, up to 8 limbs)
+    // it moved the time per layer by 4 to 6% on average, at best 100 inputs -> 40
+    // outputs: 1.96 ms with one coefficient per lane, two regions and 2 x 8 warps,
+    // 0.91 with two and one region; at worst 4% up.
     // It has to be no slower at lower levels too, down to half the limbs, where a
     // launch of few rounds of tiles may end in a nearly empty one (24 -> 26 at
     // 2^12: three CTAs of 4 warps an SM, quicker at 14 limbs, took 40.8 us
@@ -2082,7 +2094,7 @@ int lower_tiled(fiona_plan *p)
     ts->warps = best.W;
     ts->tile = T;
     ts->batch = best.P;
-    ts->est_cycles = best.level;
+    ts->est_cycles = best.launch;
     ts->has_const = has_const;
     ts->smem = best.smem;
     ts->ctas_per_sm = best.ctas;

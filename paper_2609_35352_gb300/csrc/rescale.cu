@@ -24,10 +24,9 @@
 // What bounds it: the FMA-heavy pipe (64-bit products, 4 cycles a warp), which
 // ncu shows 76% busy in the forward high pass and 69% in the low one, whose
 // epilogue also reads y.  Measured on GB300 (192 polys of 2^16, 12 -> 11
-// limbs): 1.728 ms with Shoup's product and one poly a low-pass CTA, 1.636 ms
-// with the two-word twiddles of ntt.cuh and four polys, 1.488 ms with their
-// tables in staging order (and N^-1, q^-1 in the same form), 1.410 ms with
-// eight polys; its HBM bytes take 0.34 ms.
+// limbs): 1.728 ms with Shoup's product and one poly a low-pass CTA, 1.410 ms with
+// the two-word twiddles of ntt.cuh, their tables in staging order and eight polys;
+// its HBM bytes take 0.34 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -86,7 +86,7 @@ __device__ __forceinline__ void settle(uint64_t &lo, uint64_t &mid, uint64_t &hi
 }
 
 // acc (lo, hi) += a * b, full 128-bit product, carry chained (the direct kernel's
-// form: it waits for memory, and the middle words of mac() below cost it more
+// form: it waits for memory, and the middle words of mac() above cost it more
 // registers than the multiplications save: the 64-ciphertext sum 0.338 ms
 // against 0.310 on GB300)
 __device__ __forceinline__ void mac128(uint64_t &lo, uint64_t &hi, uint64_t a, uint64_t b)

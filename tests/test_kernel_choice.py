@@ -35,8 +35,8 @@ def test_direct_kernel(n_in, n_out, L, bits, signed, direct):
 
 # at N = 2^12 and 3 limbs, the inputs up to which a layer of n outputs is direct:
 # one group a term (a batch of four each on the tiled kernel), one group an output
-SMALL = {(True, 50): {2: 4, 3: 7, 4: 9, 6: 16}, (False, 50): {3: 4, 4: 6, 6: 8, 8: 8, 12: 12, 16: 14},
-         (False, 60): {2: 7, 3: 8, 4: 8, 6: 16, 8: 16, 12: 24}}
+SMALL = {(True, 50): {2: 7, 3: 9, 4: 13, 6: 21}, (False, 50): {3: 6, 4: 7, 6: 10, 8: 10, 12: 13, 16: 17},
+         (False, 60): {2: 7, 3: 9, 4: 9, 6: 19, 8: 17, 12: 25}}
 
 
 @pytest.mark.parametrize("per_term,bits,n_out", [(*k, n) for k, v in SMALL.items() for n in v])
@@ -50,7 +50,7 @@ def test_small_launches(per_term, bits, n_out):
 
 
 @pytest.mark.parametrize("n_in,n_out,N,bits,few,many", [(16, 16, 2048, 50, 2, 6), (24, 24, 4096, 50, 1, 6),
-                                                        (7, 7, 65536, 50, 1, 8), (11, 11, 65536, 60, 1, 8)])
+                                                        (7, 7, 65536, 50, 2, 8), (11, 11, 65536, 60, 2, 8)])
 def test_fewer_limbs(n_in, n_out, N, bits, few, many):
     """The choice goes by the limbs of a launch: direct for few of them."""
     assert stats(n_in, n_out, N=N, L=few, bits=bits)["kernel"] == F.FIONA_KERNEL_DIRECT
