@@ -68,7 +68,7 @@ typedef enum fiona_status {
     FIONA_ERR_CUDA = -5,    /* a CUDA runtime call failed (launch, copy, device) */
     FIONA_ERR_RANGE = -6,   /* fiona_check_residues found a residue >= q_l */
     FIONA_ERR_NODEVICE = -7,/* evaluation requested on a validation-only context */
-    FIONA_ERR_TIMEOUT = -8, /* a kernel gave up waiting for its own copies (see fiona_device_check) */
+    FIONA_ERR_TIMEOUT = -8, /* a kernel gave up waiting for its own work (see fiona_device_check) */
     FIONA_ERR_INTERNAL = -9 /* a lowered schedule failed its own consistency check (a library bug) */
 } fiona_status;
 
@@ -472,8 +472,8 @@ int fiona_check_residues(const fiona_ctx *ctx, void *cuda_stream, const uint64_t
                          uint64_t count);
 
 /* Report kernel-side failures of earlier calls on this context:
- * synchronises `cuda_stream`, then returns FIONA_ERR_TIMEOUT if a tiled
- * kernel gave up waiting for its bulk copies or its tensor-core contraction
+ * synchronises `cuda_stream`, then returns FIONA_ERR_TIMEOUT if a tiled or
+ * matrix kernel gave up waiting for its copies, digits or tensor-core products
  * (every such wait is bounded; the CTA then stops: the outputs of that
  * evaluation are undefined, the context stays usable), FIONA_ERR_RANGE if an encoding met a
  * coefficient out of range (fiona_ckks_embed), FIONA_ERR_CUDA on a CUDA

@@ -740,7 +740,7 @@ extern "C" int fiona_device_check(const fiona_ctx *ctx, void *stream)
     if (e == cudaSuccess) e = cudaMemcpy(&flag, ctx->d_kerr, sizeof(int), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && flag) e = cudaMemset(ctx->d_kerr, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "device_check");
-    if (flag & 1) return set_error(FIONA_ERR_TIMEOUT, "a kernel gave up waiting for its bulk copies");
+    if (flag & 1) return set_error(FIONA_ERR_TIMEOUT, "a kernel gave up waiting for its copies or tensor-core products");
     if (flag & 2) return set_error(FIONA_ERR_RANGE, "an encoded coefficient was not finite or reached 2^62");
     return FIONA_OK;
 }
